@@ -517,6 +517,8 @@ struct AdjInitArgs {
     double wpsi[Q * P];
     double eps0[Q];
     double de0[Q][NTH];
+    double ratio[Q], y0[Q], ie0[Q];  // G(w0_q) / Gmax, (eps0_q / kT)^2, 1 / (1 + exp((eps0_q - mu) / kT))
+    FdInv fd;                        // the sampler's table (pgc_fd.cuh)
     double mu, kT, hvF;
 };
 
@@ -539,14 +541,24 @@ k_adj_init(const __grid_constant__ AdjArgs<P, Q, R> a, const __grid_constant__ A
             ly[h] = (double)a.lam[(int64_t)(P + h) * a.ld + i];
         }
         for (int q = 0; q < Q; ++q) {
+            // d|k|/d eps0 with deps/deps0 = rho(eps0)(1-u)/rho(eps), rho(e) = e / (1 + exp((e-mu)/kT))
             const double e0 = ia.eps0[q];
-            const double eps = fd_inverse(e0, ia.mu, ia.kT, ue);
-            const double rr2 = eps * eps - e0 * e0;
-            if (!(rr2 > 0.0)) continue;
-            const double km = sqrt(rr2) / ia.hvF;
-            auto rho = [&](double e) { return e / (1.0 + exp(fmin((e - ia.mu) / ia.kT, 700.0))); };
-            const double deps = rho(e0) * (1.0 - ue) / rho(eps);
-            const double dkm = (eps * deps - e0) / (ia.hvF * ia.hvF * km);
+            double dkm;
+            if (ia.fd.tab) {
+                double E;
+                const double y2 = fd_Y<true>(ia.fd, (1.0 - ue) * ia.ratio[q], &E) - ia.y0[q];
+                if (!(y2 > 0.0)) continue;
+                const double km = sqrt(y2) * (ia.kT / ia.hvF);
+                dkm = e0 * ((1.0 - ue) * (E * ia.ie0[q]) - 1.0) / (ia.hvF * ia.hvF * km);
+            } else {
+                const double eps = fd_inverse(e0, ia.mu, ia.kT, ue);
+                const double rr2 = eps * eps - e0 * e0;
+                if (!(rr2 > 0.0)) continue;
+                const double km = sqrt(rr2) / ia.hvF;
+                auto rho = [&](double e) { return e / (1.0 + exp(fmin((e - ia.mu) / ia.kT, 700.0))); };
+                const double deps = rho(e0) * (1.0 - ue) / rho(eps);
+                dkm = (eps * deps - e0) / (ia.hvF * ia.hvF * km);
+            }
             double mx = 0.0, my = 0.0;
 #pragma unroll
             for (int h = 0; h < P; ++h) { mx += ia.wpsi[q * P + h] * lx[h]; my += ia.wpsi[q * P + h] * ly[h]; }
@@ -623,6 +635,15 @@ public:
         ia_.mu = t.mu;
         ia_.kT = t.kT;
         ia_.hvF = t.hvF;
+        if (b.fdtab) {   // written by the sampling of the context (the adjoint starts from its sampled state)
+            ia_.fd = fd_plan(ia_.eps0, Q, t.mu, t.kT, ia_.ratio);
+            if (ia_.fd.n > 0) ia_.fd.tab = b.fdtab;
+            for (int q = 0; q < Q; ++q) {
+                const double w0 = ia_.eps0[q] / t.kT;
+                ia_.y0[q] = w0 * w0;
+                ia_.ie0[q] = 1.0 / (1.0 + std::exp(w0 - ia_.fd.m));
+            }
+        }
         int per_sm = 0;
         cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, k_adj_screen<P, Q, R>, 256, 0);
         grid_ = (int)std::max<int64_t>(1, std::min<int64_t>((b.N + 255) / 256, (int64_t)num_sms * std::max(per_sm, 1)));

@@ -23,6 +23,7 @@
 #pragma once
 
 #include "pgc_device.cuh"
+#include "pgc_fd.cuh"
 
 namespace pgc {
 
@@ -1260,6 +1261,8 @@ template <int P, int Q>
 struct InitArgs {
     double wpsi[Q * P];
     double eps0[Q];
+    double ratio[Q], y0[Q];   // G(w0_q) / Gmax and (eps0_q / kT)^2 (the table of pgc_fd.cuh)
+    FdInv fd;
     double mu, kT, hvF;
     double dhalf[P];   // Strang: the stored state leads by half a drift (x coefficients)
     int32_t strang;
@@ -1267,35 +1270,41 @@ struct InitArgs {
     uint32_t key0, key1, stream_id;
 };
 
+// Every node's |k| lies along the particle's one angle, so |k| is projected and the coefficients are
+// its projection times (cos, sin): P multiply-adds per node instead of 2P.
 template <int P, int Q, typename R>
 __global__ void __launch_bounds__(128)
 k_init(const __grid_constant__ InitArgs<P, Q> ia, R *khat)
 {
+    const double kw = ia.kT / ia.hvF;
     for (int64_t i = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; i < ia.N; i += (int64_t)gridDim.x * blockDim.x) {
         const U4 r = philox4x32_10((uint32_t)i, ia.stream_id, 0u, 0x10000u, ia.key0, ia.key1);
         const double ue = u01<double>(r.x), uth = u01<double>(r.y);
         double s, c;
         sincos(2.0 * kPi * uth, &s, &c);
-        double hx[P], hy[P];
+        double hk[P];
 #pragma unroll
-        for (int h = 0; h < P; ++h) { hx[h] = 0.0; hy[h] = 0.0; }
+        for (int h = 0; h < P; ++h) hk[h] = 0.0;
 #pragma unroll 1
         for (int q = 0; q < Q; ++q) {
-            const double e0 = ia.eps0[q];
-            const double eps = fd_inverse(e0, ia.mu, ia.kT, ue);
-            const double rr = eps * eps - e0 * e0;
-            const double km = (rr > 0.0) ? sqrt(rr) / ia.hvF : 0.0;
-            const double kx = km * c, ky = km * s;
-#pragma unroll
-            for (int h = 0; h < P; ++h) {
-                hx[h] += ia.wpsi[q * P + h] * kx;
-                hy[h] += ia.wpsi[q * P + h] * ky;
+            double km;
+            if (ia.fd.tab) {
+                const double rr = fd_Y<false>(ia.fd, (1.0 - ue) * ia.ratio[q], nullptr) - ia.y0[q];
+                km = (rr > 0.0) ? sqrt(rr) * kw : 0.0;
+            } else {
+                const double e0 = ia.eps0[q];
+                const double eps = fd_inverse(e0, ia.mu, ia.kT, ue);
+                const double rr = eps * eps - e0 * e0;
+                km = (rr > 0.0) ? sqrt(rr) / ia.hvF : 0.0;
             }
+#pragma unroll
+            for (int h = 0; h < P; ++h) hk[h] += ia.wpsi[q * P + h] * km;
         }
 #pragma unroll
         for (int h = 0; h < P; ++h) {
-            khat[(int64_t)h * ia.ld + i] = (R)(ia.strang ? hx[h] + ia.dhalf[h] : hx[h]);
-            khat[(int64_t)(P + h) * ia.ld + i] = (R)hy[h];
+            const double hx = hk[h] * c, hy = hk[h] * s;
+            khat[(int64_t)h * ia.ld + i] = (R)(ia.strang ? hx + ia.dhalf[h] : hx);
+            khat[(int64_t)(P + h) * ia.ld + i] = (R)hy;
         }
     }
 }

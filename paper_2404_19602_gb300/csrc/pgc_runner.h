@@ -58,6 +58,7 @@ struct DevBuffers {
     uint32_t *marks = nullptr;      // [kMarkSlots][mark_words] collider bitmaps or nullptr (pipelined steps only)
     int64_t mark_words = 0;
     void *tables = nullptr;         // device copy of the node tables (kTableBytes) or nullptr
+    double *fdtab = nullptr;        // table of the Fermi-Dirac inverse (pgc_fd.cuh) or nullptr
     uint32_t *recon_hist = nullptr; // [Nk*Nk]
     uint32_t key0 = 0, key1 = 0, stream_id = 0;
 };

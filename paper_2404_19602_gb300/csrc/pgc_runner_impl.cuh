@@ -109,6 +109,15 @@ public:
 
     cudaError_t init_sample(cudaStream_t s) override
     {
+        if (b_.fdtab) {
+            init_.fd = fd_plan(init_.eps0, Q, init_.mu, init_.kT, init_.ratio);
+            for (int q = 0; q < Q; ++q) { const double w0 = init_.eps0[q] / init_.kT; init_.y0[q] = w0 * w0; }
+            if (init_.fd.n > 0) {
+                k_fd_table<<<(init_.fd.n + 31) / 32, 32, 0, s>>>(init_.fd, b_.fdtab);
+                count_launch();
+                init_.fd.tab = b_.fdtab;
+            }
+        }
         int blocks = (int)std::min<int64_t>((b_.N + 127) / 128, 8192);
         k_init<P, Q, R><<<blocks, 128, 0, s>>>(init_, args_.khat);
         count_launch();
