@@ -55,6 +55,7 @@ struct BatchArgs {
     uint32_t *done;            // phase-2 block completion counter
     int32_t moments_every;
     int32_t win_r0, use_win;
+    R kk_in;                   // as in StepArgs, common to the cases (the batched kernels run the Lie splitting)
     int32_t rec_len;
     double vF_ms;
 };
@@ -82,7 +83,8 @@ k_phase1_batch(const __grid_constant__ BatchArgs<P, Q, R> a)
     __shared__ typename MomAcc<R>::T smom[NW][Q * 3];
     __shared__ int64_t stile[kBatchMaxCases + 1];
     __shared__ __align__(16) uint32_t snd[(sizeof(Nodes<P, Q, R>) + 3) / 4];
-    extern __shared__ uint32_t swin[];
+    __shared__ uint32_t s_aside[sizeof(R) == 4 ? NW : 1][sizeof(R) == 4 ? AsideList<PPT>::cap : 1];
+    extern __shared__ __align__(16) uint32_t swin[];
     const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
     const int64_t step = *a.d_step;
     const int nxt = (int)((step + 1) % kHistBufs), clr = (int)((step + 2) % kHistBufs);
@@ -92,7 +94,8 @@ k_phase1_batch(const __grid_constant__ BatchArgs<P, Q, R> a)
     __syncthreads();
     const int64_t NN = (int64_t)a.ph.Nk * a.ph.Nk;
     const int64_t helems = (int64_t)Q * NN;
-    int cur = -1;
+    int cur = -1, n_aside = 0;
+    uint32_t *aside = s_aside[sizeof(R) == 4 ? warp : 0];
     unsigned int oog = 0u;
     for (int64_t tile = blockIdx.x; tile < a.ntiles; tile += gridDim.x) {
         const int c = find_case(stile, a.ncases + 1, tile);
@@ -102,8 +105,7 @@ k_phase1_batch(const __grid_constant__ BatchArgs<P, Q, R> a)
             stage(snd, cd.nd);
             cur = c;
         }
-        if (a.use_win)
-            for (int j = threadIdx.x; j < Q * kWinWords; j += blockDim.x) swin[j] = 0u;
+        if (a.use_win) clear_window<Q, HistWin<P, Q, R>::batchW>(swin);
         if (out)
             for (int j = lane; j < Q * 3; j += 32) acc_zero(smom[warp][j]);
         // this tile's share of clearing the case's buffer of step n+2
@@ -127,10 +129,14 @@ k_phase1_batch(const __grid_constant__ BatchArgs<P, Q, R> a)
         const int64_t p0 = (tile - cd.tile0) * a.tile;
         const int64_t p1 = min(cd.N, p0 + a.tile);
         for (int64_t base = p0; base < p1; base += (int64_t)blockDim.x * PPT)
-            phase1_pass<P, Q, R, PPT>(a.ph, nd, t, base + (int64_t)threadIdx.x * PPT, swin, a.win_r0, a.use_win != 0,
-                                      out, smom[warp], oog);
+            phase1_pass<P, Q, R, HistWin<P, Q, R>::batchW, PPT>(a.ph, nd, t, base + (int64_t)threadIdx.x * PPT, swin, a.win_r0, a.use_win != 0, a.kk_in,
+                                      out, smom[warp], aside, n_aside, oog);
+        if (sizeof(R) == 4 && n_aside > 0) {
+            count_aside<P, Q, R, HistWin<P, Q, R>::batchW>(a.ph, nd, t, aside, n_aside, swin, a.win_r0, a.use_win != 0, oog);
+            n_aside = 0;
+        }
         __syncthreads();
-        if (a.use_win) flush_window<Q>(swin, t.Hnext, a.ph.Nk, a.win_r0);
+        if (a.use_win) flush_window<Q, HistWin<P, Q, R>::batchW>(swin, t.Hnext, a.ph.Nk, a.win_r0);
         if (out)
             for (int j = threadIdx.x; j < Q * 3; j += blockDim.x) {
                 double s = 0.0;
@@ -327,11 +333,13 @@ public:
         a_.d_step = sc.d_step;
         a_.done = sc.done;
         a_.moments_every = 0;
-        a_.win_r0 = proto.args().win_r0;
-        a_.use_win = proto.args().use_win;
+        constexpr int W = HistWin<P, Q, R>::batchW;
+        a_.use_win = t0.Nk >= W;
+        a_.win_r0 = window_r0(t0.Nk, W);
+        a_.kk_in = a_.use_win ? (R)window_kk(t0, W) : (R)-1;
         a_.rec_len = 1 + 4 * Q + 8;
         a_.vF_ms = t0.vF_ms;
-        win_bytes_ = a_.use_win ? (size_t)Q * kWinWords * 4 : 0;
+        win_bytes_ = a_.use_win ? HistWin<P, Q, R>::batch_bytes : 0;
         num_sms_ = num_sms;
         for (int j = 0; j < BatchPPTs<P>::n; ++j)
             if (win_bytes_) cudaFuncSetAttribute(kernel1(BatchPPTs<P>::v[j]), cudaFuncAttributeMaxDynamicSharedMemorySize, (int)win_bytes_);

@@ -27,7 +27,7 @@
 
 namespace pgc {
 
-constexpr int kPhase1Threads = 256;
+constexpr int kPhase1Threads = 256;   // threads of a streaming block (P1Threads: 512 at 36 nodes in FP32)
 constexpr int kPhase2Threads = 128;
 constexpr int kMaxGrid1 = 4096;   // block partials sized for at most this many phase-1 blocks
 constexpr int kGrid2 = 608;       // phase-2 blocks (grid-stride over the queue)
@@ -35,9 +35,29 @@ constexpr int kGrid2 = 608;       // phase-2 blocks (grid-stride over the queue)
 // were measured 1 % slower with the collider's rolled slot loops, six slower still).
 template <int P, int Q> struct Phase2Blocks { static constexpr int per_sm = 4; };
 constexpr int kGrid2Max = 5 * 152; // phase-2 partial sums are sized for this many blocks
-// Block-private histogram window of phase 1: kWin x kWin cells per node around the grid centre,
-// 16-bit counts packed two per 32-bit word in shared memory, flushed to the global histogram once
-// per block.  Cells outside the window go straight to the global histogram.
+// Block-private histogram window of the streaming kernels: W x W cells around the grid centre, in
+// shared memory, flushed to the global histogram once per block.  Two nodes share a word per cell,
+// node 2p in the low and node 2p + 1 in the high half, so that a node's increment is a constant
+// (1 or 1 << 16) and a cell's byte offset within a node pair is one multiply-add of its row and
+// column.  Cells outside the window go straight to the global histogram.
+//   36 nodes, FP32: one block of 512 threads per SM owns one window of 48 x 48 cells (166 KB).  Two
+//   blocks with 32 x 32 each (+-0.67 eV) left 2-4 % of the particles with a node outside (3/4 of
+//   the warps had such a lane) once the field had heated the ensemble; 48 x 48 (+-1 eV): 0.1 %.
+//   One-dimensional shapes: 48 x 48 up to 6 nodes (28 KB), else 40 x 40 (31 nodes 102 KB); 36 nodes
+//   FP64: 32 x 32.
+template <int P, int Q, typename R> struct HistWin {
+    static constexpr int pairs = (Q + 1) / 2;
+    static constexpr int W = (Q == 36) ? (sizeof(R) == 4 ? 48 : 32) : (Q <= 6 ? 48 : 40);
+    static constexpr size_t bytes = (size_t)pairs * W * W * 4;
+    // the batched kernel (blocks of up to 256 threads, two per SM at 36 nodes)
+    static constexpr int batchW = (Q == 36) ? (sizeof(R) == 4 ? 36 : 32) : 56;
+    static constexpr size_t batch_bytes = (size_t)pairs * batchW * batchW * 4;
+};
+// threads of a streaming block
+template <int P, int Q, typename R> struct P1Threads {
+    static constexpr int value = (Q == 36 && sizeof(R) == 4) ? 512 : kPhase1Threads;
+};
+// The window of the tensor-core streaming kernel: kWin x kWin cells per node, two columns per word.
 constexpr int kWin = 32;
 constexpr int kWinWords = kWin * kWin / 2;
 // Rotating buffers.  Histogram f^n lives in buffer n % kHistBufs: while phase 2 of step n - 1
@@ -77,6 +97,7 @@ struct Nodes {
     unsigned long long psi2[(TensorShape<P, Q>::value || sizeof(R) == 8) ? 1 : Q * P];
     unsigned long long wpsi2[(TensorShape<P, Q>::value || sizeof(R) == 8) ? 1 : Q * P];
     unsigned long long a1_2[36], b2_2[36];
+    unsigned long long lk2[sizeof(R) == 8 ? 1 : Q];   // FP32: (lkx[q], Lk)
 };
 
 template <int P, int Q, typename R>
@@ -102,6 +123,7 @@ struct StepArgs {
     int32_t out_step;        // 1: accumulate the moments of the post-step state
     int32_t win_r0;          // first row / column of the shared-memory window
     int32_t use_win;         // 1: phase 1 counts into the shared-memory window
+    R kk_in;                 // |k|^2 up to which a node value's cell lies in the window (< 0: none known to)
     // collider bitmaps (bit i of word i / 32), all optional (nullptr)
     const uint32_t *skip;    // phase 1: particles queued at step n - 1, owned by a concurrent phase 2
     uint32_t *mark;          // phase 1: set for every particle queued at step n
@@ -268,6 +290,44 @@ __device__ __forceinline__ F2 f2_fma(F2 a, unsigned long long w2, F2 c)
     return r;
 }
 
+__device__ __forceinline__ F2 f2_add(F2 a, unsigned long long b)
+{
+    F2 r;
+    asm("add.rn.f32x2 %0, %1, %2;" : "=l"(r.v) : "l"(a.v), "l"(b));
+    return r;
+}
+__device__ __forceinline__ F2 f2_mul(F2 a, F2 b)
+{
+    F2 r;
+    asm("mul.rn.f32x2 %0, %1, %2;" : "=l"(r.v) : "l"(a.v), "l"(b.v));
+    return r;
+}
+__device__ __forceinline__ F2 f2_add_rd(F2 a, F2 b)
+{
+    F2 r;
+    asm("add.rm.f32x2 %0, %1, %2;" : "=l"(r.v) : "l"(a.v), "l"(b.v));
+    return r;
+}
+
+// Byte offset, within a node pair's part of the window, of the cell of a node value inside the window
+// (the bits above 15 and the low two are not meaningful: mask with 0xfffc).  The cell is that of
+// cell_rl: the same addition and multiplication, and floor by an addition rounded down at a magnitude
+// where a float's last bit is 1 (row, 2^23) or 1/4 (column, 2^21): the low bits of the sums are then
+// row - r0 and 4 (column - r0) + fraction.  Three packed operations and a multiply-add where two
+// additions, two multiplications, two conversions, the bounds checks and the word and shift
+// arithmetic were ~20.  A particle whose |k| stays inside the window's circle at every node (kk_in, from
+// the majorant's kkmax that the screen needs anyway) takes no per-node check at all.  Measured: the
+// streaming kernel at 4e6 particles x 36 nodes 465 -> 237 us in the first 50 steps, 487 -> 260 us after
+// 3000 (one step in ten with moments); the batched kernel at 32 cases, 1.3e7 particles x 6 nodes
+// 355 -> 246 and 388 -> 269 us; instructions issued bound both.
+template <int W>
+__device__ __forceinline__ uint32_t window_code(float kx, float ky, unsigned long long lk2, F2 inv2, F2 magic2)
+{
+    const F2 s = f2_add_rd(f2_mul(f2_add(f2_pack(kx, ky), lk2), inv2), magic2);
+    return (uint32_t)s.v * (4u * W) + (uint32_t)(s.v >> 32);
+}
+__device__ __forceinline__ F2 window_magic(int r0) { return f2_pack(8388608.0f - (float)r0, 2097152.0f - (float)r0); }
+
 template <int P, int Q, typename R>
 __device__ __forceinline__ void recon_node(const Nodes<P, Q, R> &nd, int q, const R cx[P], const R cy[P],
                                            R &kx, R &ky)
@@ -286,6 +346,43 @@ __device__ __forceinline__ void recon_node(const Nodes<P, Q, R> &nd, int q, cons
         }
         kx = sx;
         ky = sy;
+    }
+}
+
+// The node values of recon_all (same operations in the same order) by a rolled loop over the rows of
+// nodes: for code that seldom runs.
+template <int P, int Q, typename R, typename F>
+__device__ __forceinline__ void recon_all_rolled(const Nodes<P, Q, R> &nd, const R cx[P], const R cy[P], F &&f)
+{
+    if constexpr (TensorShape<P, Q>::value && sizeof(R) == 4) {
+#pragma unroll 1
+        for (int q1 = 0; q1 < 6; ++q1) {
+            F2 t2[6];
+#pragma unroll
+            for (int h2 = 0; h2 < 6; ++h2) {
+                F2 s2 = f2_pack(0.f, 0.f);
+#pragma unroll
+                for (int h1 = 0; h1 + h2 <= 5; ++h1)
+                    s2 = f2_fma(f2_pack(cx[hidx2(h1, h2)], cy[hidx2(h1, h2)]), nd.a1_2[q1 * 6 + h1], s2);
+                t2[h2] = s2;
+            }
+#pragma unroll
+            for (int q2 = 0; q2 < 6; ++q2) {
+                F2 k2 = f2_pack(0.f, 0.f);
+#pragma unroll
+                for (int h2 = 0; h2 < 6; ++h2) k2 = f2_fma(t2[h2], nd.b2_2[q2 * 6 + h2], k2);
+                R kx, ky;
+                f2_unpack(k2, kx, ky);
+                f(q1 * 6 + q2, kx, ky);
+            }
+        }
+    } else {
+#pragma unroll 1
+        for (int q = 0; q < Q; ++q) {
+            R kx, ky;
+            recon_node(nd, q, cx, cy, kx, ky);
+            f(q, kx, ky);
+        }
     }
 }
 
@@ -410,9 +507,10 @@ __device__ __forceinline__ void observe_fast(const Phys<float> &ph, float kx, fl
 // ------------------------------------------------------------------------------------------
 template <int P> struct Phase1PPT { static constexpr int value = (P <= 8) ? 4 : 1; };
 // resident blocks per SM the streaming kernels are compiled for: three for the small FP32
-// shapes, two (more registers, no spills) for 36 nodes and for FP64
+// shapes, two (more registers, no spills) for the large shapes and for FP64; one block of 512
+// threads for 36 nodes in FP32 (the same 128 registers, one window per SM)
 template <int P, int Q, typename R> struct kPhase1MinBlocks {
-    static constexpr int value = (P * Q > 64 || sizeof(R) == 8) ? 2 : 3;
+    static constexpr int value = (Q == 36 && sizeof(R) == 4) ? 1 : (P * Q > 64 || sizeof(R) == 8) ? 2 : 3;
 };
 
 template <typename R, int PPT>
@@ -469,13 +567,48 @@ struct P1Target {
     uint32_t *mark = nullptr;        // optional: bitmap of the particles queued here
 };
 
+// The particles of a warp with a node value outside the circle of the window (kk_in), put aside in
+// shared memory: a rolled pass over their nodes for one lane costs a warp as much as for 32, so they
+// are taken 32 at a time (FP32 kernels; at most 31 stay between passes).
+template <int PPT> struct AsideList { static constexpr int cap = 32 * (PPT + 1); };
+
+// Counts the histogram cells of n <= 32 such particles (one per lane) from their stored state.
+template <int P, int Q, typename R, int W>
+__device__ __forceinline__ void count_aside(const Phys<R> &ph, const Nodes<P, Q, R> &nd, const P1Target<R> &t, const uint32_t *list,
+                                            int n, uint32_t *swin, int win_r0, bool use_win, unsigned int &oog)
+{
+    const int lane = threadIdx.x & 31;
+    const int64_t NN = (int64_t)ph.Nk * ph.Nk;
+    __syncwarp();   // the list and the drifted coefficients, written by other lanes
+    if (lane < n) {
+        const int64_t i = list[lane];
+        R cx[P], cy[P];
+#pragma unroll
+        for (int h = 0; h < P; ++h) {
+            cx[h] = t.khat[(int64_t)h * t.ld + i];
+            cy[h] = t.khat[(int64_t)(P + h) * t.ld + i];
+        }
+        recon_all_rolled(nd, cx, cy, [&](int q, R kx, R ky) {
+            int r, l;
+            if (!cell_rl(ph, nd.lkx[q], kx, ky, r, l)) { ++oog; return; }
+            const int rr = r - win_r0, ll = l - win_r0;
+            if (use_win && (unsigned)rr < (unsigned)W && (unsigned)ll < (unsigned)W)
+                atomicAdd(&swin[(q >> 1) * (W * W) + rr * W + ll], 1u << ((q & 1) << 4));
+            else
+                atomicAdd(&t.Hnext[(int64_t)q * NN + r * ph.Nk + l], 1u);
+        });
+    }
+    __syncwarp();   // the list may be written again
+}
+
 // One pass of a block over blockDim * PPT consecutive particles starting at i0 + threadIdx*PPT:
 // drift, reconstruction, flight-time screen, histogram (window or global), queue, moments.
 // (PPT particles per thread; i0 a multiple of PPT.)
-template <int P, int Q, typename R, int PPT = Phase1PPT<P>::value>
+template <int P, int Q, typename R, int W = HistWin<P, Q, R>::W, int PPT = Phase1PPT<P>::value>
 __device__ __forceinline__ void phase1_pass(const Phys<R> &ph, const Nodes<P, Q, R> &nd, const P1Target<R> &t,
-                                            int64_t i0, uint32_t *swin, int win_r0, bool use_win, bool out_step,
-                                            typename MomAcc<R>::T *smom_warp, unsigned int &oog)
+                                            int64_t i0, uint32_t *swin, int win_r0, bool use_win, R kk_in, bool out_step,
+                                            typename MomAcc<R>::T *smom_warp, uint32_t *aside, int &n_aside,
+                                            unsigned int &oog)
 {
     const int lane = threadIdx.x & 31;
     const int64_t NN = (int64_t)ph.Nk * ph.Nk;
@@ -518,30 +651,54 @@ __device__ __forceinline__ void phase1_pass(const Phys<R> &ph, const Nodes<P, Q,
     for (int e = 0; e < PPT; ++e) {
         const int64_t i = i0 + e;
         finished[e] = false;
-        bool maybe = false;
+        bool maybe = false, put_aside = false;
         if (any && i < t.N && !((skipbits >> e) & 1u)) {
             // reconstruction, cells and the bound on the majorant
-            int rl[Q];   // cell (row << 16) | column; -1 outside the grid
+            uint32_t cell[Q];   // FP32: window_code; FP64: (row << 16) | column, ~0 outside the grid
             R kkmax = (R)0;
+            F2 inv2, magic2;
+            if constexpr (sizeof(R) == 4) { inv2 = f2_pack(ph.inv_dk, ph.inv_dk); magic2 = window_magic(win_r0); }
             recon_all(nd, cx[e], cy[e], [&](int q, R kx, R ky) {
-                int r, l;
-                rl[q] = cell_rl(ph, nd.lkx[q], kx, ky, r, l) ? ((r << 16) | l) : -1;
+                if constexpr (sizeof(R) == 4) {
+                    cell[q] = window_code<W>(kx, ky, nd.lk2[q], inv2, magic2);
+                } else {
+                    int r, l;
+                    cell[q] = cell_rl(ph, nd.lkx[q], kx, ky, r, l) ? (uint32_t)((r << 16) | l) : ~0u;
+                }
                 kkmax = fmax(kkmax, knorm2(kx, ky));
             });
             const U4 r = philox4x32_10((uint32_t)i, t.stream_id, t.step, 0u, t.key0, t.key1);
             maybe = screen_maybe(ph, nd, kkmax, r.x);
             if (!maybe) {
                 finished[e] = true;
+                if constexpr (sizeof(R) == 4) {
+                    if (kkmax <= kk_in) {   // every node value lies in the window
 #pragma unroll (kUnrollQ ? Q : 1)
-                for (int q = 0; q < Q; ++q) {
-                    if (rl[q] < 0) { ++oog; continue; }
-                    const int r = rl[q] >> 16, l = rl[q] & 0xffff;
-                    const int rr = r - win_r0, ll = l - win_r0;
-                    if (use_win && (unsigned)rr < (unsigned)kWin && (unsigned)ll < (unsigned)kWin)
-                        atomicAdd(&swin[q * kWinWords + rr * (kWin / 2) + (ll >> 1)], 1u << ((ll & 1) << 4));
-                    else
-                        atomicAdd(&t.Hnext[(int64_t)q * NN + r * ph.Nk + l], 1u);
+                        for (int q = 0; q < Q; ++q)
+                            atomicAdd(reinterpret_cast<uint32_t *>(reinterpret_cast<char *>(swin + (q >> 1) * (W * W)) + (cell[q] & 0xfffcu)),
+                                      (q & 1) ? 0x10000u : 1u);
+                    } else {
+                        put_aside = true;
+                    }
+                } else {
+#pragma unroll (kUnrollQ ? Q : 1)
+                    for (int q = 0; q < Q; ++q) {
+                        if (cell[q] == ~0u) { ++oog; continue; }
+                        const int r = (int)(cell[q] >> 16), l = (int)(cell[q] & 0xffffu);
+                        const int rr = r - win_r0, ll = l - win_r0;
+                        if (use_win && (unsigned)rr < (unsigned)W && (unsigned)ll < (unsigned)W)
+                            atomicAdd(&swin[(q >> 1) * (W * W) + rr * W + ll], 1u << ((q & 1) << 4));
+                        else
+                            atomicAdd(&t.Hnext[(int64_t)q * NN + r * ph.Nk + l], 1u);
+                    }
                 }
+            }
+        }
+        if constexpr (sizeof(R) == 4) {
+            const unsigned int am = __ballot_sync(0xffffffffu, put_aside);
+            if (am) {
+                if (put_aside) aside[n_aside + __popc(am & ((1u << lane) - 1u))] = (uint32_t)i;
+                n_aside += __popc(am);
             }
         }
         // colliders go to the queue (warp-aggregated append)
@@ -616,11 +773,45 @@ __device__ __forceinline__ void phase1_pass(const Phys<R> &ph, const Nodes<P, Q,
             }
         }
     }
+    if constexpr (sizeof(R) == 4) {
+        while (n_aside >= 32) {
+            n_aside -= 32;
+            count_aside<P, Q, R, W>(ph, nd, t, aside + n_aside, 32, swin, win_r0, use_win, oog);
+        }
+    }
 }
 
-// Add a block's shared-memory window to the global histogram: one add per non-empty cell.
-template <int Q>
+// Clear a block's window; add it to the global histogram, one add per non-empty cell and node (the
+// words of the window are mostly empty: four are looked at per load).
+template <int Q, int W>
+__device__ __forceinline__ void clear_window(uint32_t *swin)
+{
+    for (int j = threadIdx.x; j < (Q + 1) / 2 * (W * W / 4); j += blockDim.x)
+        reinterpret_cast<uint4 *>(swin)[j] = make_uint4(0u, 0u, 0u, 0u);
+}
+
+template <int Q, int W>
 __device__ __forceinline__ void flush_window(const uint32_t *swin, uint32_t *Hnext, int Nk, int win_r0)
+{
+    static_assert(W % 4 == 0, "four cells of a row per load");
+    const int64_t NN = (int64_t)Nk * Nk;
+    for (int j = threadIdx.x; j < (Q + 1) / 2 * (W * W / 4); j += blockDim.x) {
+        const uint4 v4 = reinterpret_cast<const uint4 *>(swin)[j];
+        if (!(v4.x | v4.y | v4.z | v4.w)) continue;
+        const int p = j / (W * W / 4), w = j % (W * W / 4);
+        uint32_t *base = Hnext + (int64_t)(2 * p) * NN + (int64_t)(w / (W / 4) + win_r0) * Nk + 4 * (w % (W / 4)) + win_r0;
+        const uint32_t v[4] = {v4.x, v4.y, v4.z, v4.w};
+#pragma unroll
+        for (int c = 0; c < 4; ++c) {
+            if (v[c] & 0xffffu) atomicAdd(base + c, v[c] & 0xffffu);
+            if (v[c] >> 16) atomicAdd(base + NN + c, v[c] >> 16);
+        }
+    }
+}
+
+// The window of the tensor-core streaming kernel.
+template <int Q>
+__device__ __forceinline__ void flush_window_tc(const uint32_t *swin, uint32_t *Hnext, int Nk, int win_r0)
 {
     const int64_t NN = (int64_t)Nk * Nk;
     for (int j = threadIdx.x; j < Q * kWinWords; j += blockDim.x) {
@@ -641,12 +832,14 @@ template <int P, int Q, typename R>
 __device__ __forceinline__ void phase1_block(const StepArgs<P, Q, R> &a, int bid, int nb, uint32_t *swin)
 {
     constexpr int PPT = Phase1PPT<P>::value;
-    constexpr int NW = kPhase1Threads / 32;
+    constexpr int NW = P1Threads<P, Q, R>::value / 32;
     __shared__ typename MomAcc<R>::T smom[NW][Q * 3];
     __shared__ uint32_t s_tile;
+    __shared__ uint32_t s_aside[sizeof(R) == 4 ? NW : 1][sizeof(R) == 4 ? AsideList<PPT>::cap : 1];
     const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
-    if (a.use_win)
-        for (int j = threadIdx.x; j < Q * kWinWords; j += blockDim.x) swin[j] = 0u;
+    uint32_t *aside = s_aside[sizeof(R) == 4 ? warp : 0];
+    int n_aside = 0;
+    if (a.use_win) clear_window<Q, HistWin<P, Q, R>::W>(swin);
     if (a.out_step)
         for (int j = lane; j < Q * 3; j += 32) acc_zero(smom[warp][j]);
     __syncthreads();
@@ -681,11 +874,11 @@ __device__ __forceinline__ void phase1_block(const StepArgs<P, Q, R> &a, int bid
     // flush (block-uniform; with the tile counter a block may take any number of tiles).
     int64_t since_flush = 0;
     auto guard_window = [&]() {
-        if (a.use_win && since_flush + tile > 65535) {
+        if (a.use_win && since_flush + tile + blockDim.x > 65535) {   // (blockDim.x: particles put aside before the flush)
             __syncthreads();
-            flush_window<Q>(swin, a.Hnext, a.ph.Nk, a.win_r0);
+            flush_window<Q, HistWin<P, Q, R>::W>(swin, a.Hnext, a.ph.Nk, a.win_r0);
             __syncthreads();
-            for (int j = threadIdx.x; j < Q * kWinWords; j += blockDim.x) swin[j] = 0u;
+            clear_window<Q, HistWin<P, Q, R>::W>(swin);
             __syncthreads();
             since_flush = 0;
         }
@@ -701,19 +894,21 @@ __device__ __forceinline__ void phase1_block(const StepArgs<P, Q, R> &a, int bid
             if (tl >= ntiles) break;
             guard_window();
             phase1_pass<P, Q, R>(a.ph, a.nd, t, tl * tile + (int64_t)threadIdx.x * PPT, swin, a.win_r0,
-                                 a.use_win != 0, a.out_step != 0, smom[warp], oog);
+                                 a.use_win != 0, a.kk_in, a.out_step != 0, smom[warp], aside, n_aside, oog);
         }
     } else {
         for (int64_t base = (int64_t)bid * tile; base < a.N; base += (int64_t)nb * tile) {
             guard_window();
-            phase1_pass<P, Q, R>(a.ph, a.nd, t, base + (int64_t)threadIdx.x * PPT, swin, a.win_r0, a.use_win != 0,
-                                 a.out_step != 0, smom[warp], oog);
+            phase1_pass<P, Q, R>(a.ph, a.nd, t, base + (int64_t)threadIdx.x * PPT, swin, a.win_r0, a.use_win != 0, a.kk_in,
+                                 a.out_step != 0, smom[warp], aside, n_aside, oog);
         }
     }
+    if (sizeof(R) == 4 && n_aside > 0)
+        count_aside<P, Q, R, HistWin<P, Q, R>::W>(a.ph, a.nd, t, aside, n_aside, swin, a.win_r0, a.use_win != 0, oog);
     oog = warp_sum(oog);
     if (lane == 0 && oog) atomicAdd(&a.counters[4], (unsigned long long)oog);
     __syncthreads();
-    if (a.use_win) flush_window<Q>(swin, a.Hnext, a.ph.Nk, a.win_r0);
+    if (a.use_win) flush_window<Q, HistWin<P, Q, R>::W>(swin, a.Hnext, a.ph.Nk, a.win_r0);
     if (a.out_step) {
         for (int j = threadIdx.x; j < Q * 3; j += blockDim.x) {
             double s = 0.0;
@@ -725,10 +920,10 @@ __device__ __forceinline__ void phase1_block(const StepArgs<P, Q, R> &a, int bid
 }
 
 template <int P, int Q, typename R>
-__global__ void __launch_bounds__(kPhase1Threads, kPhase1MinBlocks<P, Q, R>::value)
+__global__ void __launch_bounds__(P1Threads<P, Q, R>::value, kPhase1MinBlocks<P, Q, R>::value)
 k_phase1(const __grid_constant__ StepArgs<P, Q, R> a)
 {
-    extern __shared__ uint32_t swin[];   // [Q][kWinWords] when a.use_win
+    extern __shared__ __align__(16) uint32_t swin[];   // HistWin when a.use_win
     phase1_block<P, Q, R>(a, blockIdx.x, gridDim.x, swin);
 }
 
@@ -1197,10 +1392,10 @@ k_phase2(const __grid_constant__ StepArgs<P, Q, R> a)
 // counter, skipping the particles queued at step n - 1).  The two roles touch disjoint particles;
 // shared buffers are only added to (histograms, queue of step n, bitmap of step n).
 template <int P, int Q, typename R>
-__global__ void __launch_bounds__(kPhase1Threads, kPhase1MinBlocks<P, Q, R>::value)
+__global__ void __launch_bounds__(P1Threads<P, Q, R>::value, kPhase1MinBlocks<P, Q, R>::value)
 k_step(const __grid_constant__ StepArgs<P, Q, R> a1, const __grid_constant__ StepArgs<P, Q, R> a2, int nb2)
 {
-    extern __shared__ uint32_t swin[];   // phase 1: histogram window; phase 2: projection area
+    extern __shared__ __align__(16) uint32_t swin[];   // phase 1: histogram window; phase 2: projection area
     if ((int)blockIdx.x < nb2) phase2_block<P, Q, R, true>(a2, blockIdx.x, nb2, reinterpret_cast<R *>(swin));
     else phase1_block<P, Q, R>(a1, blockIdx.x - nb2, gridDim.x - nb2, swin);
 }
@@ -1210,10 +1405,10 @@ k_step(const __grid_constant__ StepArgs<P, Q, R> a1, const __grid_constant__ Ste
 // Used after the initial sampling and after a state upload.
 // ------------------------------------------------------------------------------------------
 template <int P, int Q, typename R>
-__global__ void __launch_bounds__(kPhase1Threads)
+__global__ void __launch_bounds__(P1Threads<P, Q, R>::value)
 k_observe(const __grid_constant__ StepArgs<P, Q, R> a)
 {
-    constexpr int NW = kPhase1Threads / 32;
+    constexpr int NW = P1Threads<P, Q, R>::value / 32;
     __shared__ double smom[NW][Q * 3];
     const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
     for (int j = lane; j < Q * 3; j += 32) smom[warp][j] = 0.0;

@@ -166,7 +166,7 @@ k_phase1_tc(const __grid_constant__ StepArgs<P, Q, float> a, int mode)
     for (int64_t it = 0; it < iters; ++it) {
         if (use_win && since_flush + kTcThreads > 65535) {   // CTA-uniform (see phase1_block)
             __syncthreads();
-            flush_window<Q>(swin, a.Hnext, ph.Nk, a.win_r0);
+            flush_window_tc<Q>(swin, a.Hnext, ph.Nk, a.win_r0);
             __syncthreads();
             for (int j = tid; j < Q * kWinWords; j += kTcThreads) swin[j] = 0u;
             __syncthreads();
@@ -349,7 +349,7 @@ k_phase1_tc(const __grid_constant__ StepArgs<P, Q, float> a, int mode)
     if (lane == 0 && oog) atomicAdd(&a.counters[4], (unsigned long long)oog);
     if (tc_err) atomicOr(&a.counters[6], 1ull);
     __syncthreads();
-    if (use_win) flush_window<Q>(swin, a.Hnext, ph.Nk, a.win_r0);
+    if (use_win) flush_window_tc<Q>(swin, a.Hnext, ph.Nk, a.win_r0);
     if (out_step)
         for (int j = tid; j < Q * 3; j += kTcThreads) {
             double s = 0.0;

@@ -13,6 +13,19 @@
 
 namespace pgc {
 
+// First row and column of a window of W x W cells around k = 0, and |k|^2 of the largest circle
+// about k = 0 whose cells all lie in it: 0.01 cell is left for the rounding of the cell (at most
+// 5e-4 cells), and the largest Strang shift of a node; -1 if there is none.
+inline int window_r0(int Nk, int W) { return std::max(0, Nk / 2 - W / 2); }
+inline double window_kk(const HostTables &t, int W)
+{
+    const int r0 = window_r0(t.Nk, W);
+    double xs = 0.0;
+    for (double x : t.xs) xs = std::max(xs, std::fabs(x));
+    const double rad = (std::min(0.5 * t.Nk - r0, r0 + W - 0.5 * t.Nk) - 0.01) * t.dk - xs;
+    return rad > 0.0 ? rad * rad * (1.0 - 1e-6) : -1.0;
+}
+
 template <int P, int Q, typename R>
 class RunnerT final : public Runner {
 public:
@@ -27,6 +40,13 @@ public:
             nd.dq[q] = (R)t.dq[q];
             nd.lkx[q] = (R)(t.Lk - t.xs[q]);   // Lie: the grid's Lk itself
             nd.xs[q] = (R)t.xs[q];
+            if constexpr (sizeof(R) == 4) {   // (lkx, Lk) as the two-lane operand of window_code
+                const float lo = nd.lkx[q], hi = (float)t.Lk;
+                uint32_t ul, uh;
+                std::memcpy(&ul, &lo, 4);
+                std::memcpy(&uh, &hi, 4);
+                nd.lk2[q] = ((unsigned long long)uh << 32) | ul;
+            }
         }
         nd.eps0_max = (R)t.eps0_max;
         if constexpr (TensorShape<P, Q>::value) {
@@ -78,28 +98,29 @@ public:
         // phase-1 grid: enough resident blocks to fill the GPU, PPT particles per thread; the
         // shared-memory histogram window lies inside the grid (its 16-bit cells are flushed by
         // the block before they could overflow, at any N)
-        constexpr int PPT = Phase1PPT<P>::value;
-        win_bytes_ = (size_t)Q * kWinWords * 4;
-        args_.win_r0 = std::max(0, t.Nk / 2 - kWin / 2);
-        bool win = t.Nk >= kWin && win_bytes_ <= 160 * 1024;
+        constexpr int PPT = Phase1PPT<P>::value, T1 = P1Threads<P, Q, R>::value, W = HistWin<P, Q, R>::W;
+        win_bytes_ = HistWin<P, Q, R>::bytes;
+        args_.win_r0 = window_r0(t.Nk, W);
+        bool win = t.Nk >= W;
         if (win && (cudaFuncSetAttribute(k_phase1<P, Q, R>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)win_bytes_) != cudaSuccess ||
                     !fused_attr())) {
             cudaGetLastError();
             win = false;
         }
         int per_sm = 0;
-        cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, k_phase1<P, Q, R>, kPhase1Threads, win ? win_bytes_ : 0);
+        cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, k_phase1<P, Q, R>, T1, win ? win_bytes_ : 0);
         per_sm = std::max(per_sm, 1);
-        const int64_t need = (b.N + (int64_t)kPhase1Threads * PPT - 1) / ((int64_t)kPhase1Threads * PPT);
+        const int64_t need = (b.N + (int64_t)T1 * PPT - 1) / ((int64_t)T1 * PPT);
         grid1_ = (int)std::max<int64_t>(1, std::min<int64_t>({need, (int64_t)num_sms * per_sm, (int64_t)kMaxGrid1}));
         args_.use_win = win ? 1 : 0;
         if (!win) win_bytes_ = 0;
+        args_.kk_in = win ? (R)window_kk(t, W) : (R)-1;
         // phase 2: one resident wave (its work is one latency-bound collision chain per group)
         int per_sm2 = 0;
         cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm2, k_phase2<P, Q, R, true>, kPhase2Threads, 0);
         grid2_ = std::max(1, std::min(P * Q > 64 ? kGrid2Max : kGrid2, num_sms * std::max(per_sm2, 1)));
         // the fused step kernel: as many collider groups as grid2_ blocks of phase 2 carry
-        grid2f_ = std::max(1, grid2_ * kPhase2Threads / kPhase1Threads);
+        grid2f_ = std::max(1, grid2_ * kPhase2Threads / T1);
     }
 
     int grid1() const override { return grid1_; }
@@ -129,7 +150,7 @@ public:
         StepArgs<P, Q, R> a = args_;
         a.Hnext = b_.hist + (int64_t)buf * b_.hist_stride;
         a.out_step = 1;
-        k_observe<P, Q, R><<<grid1_, kPhase1Threads, 0, s>>>(a);
+        k_observe<P, Q, R><<<grid1_, P1Threads<P, Q, R>::value, 0, s>>>(a);
         count_launch();
         return cudaGetLastError();
     }
@@ -140,7 +161,7 @@ public:
         a.Hnext = hist;
         a.part1 = part;
         a.out_step = 1;
-        k_observe<P, Q, R><<<grid1_, kPhase1Threads, 0, s>>>(a);
+        k_observe<P, Q, R><<<grid1_, P1Threads<P, Q, R>::value, 0, s>>>(a);
         count_launch();
         return cudaGetLastError();
     }
@@ -184,7 +205,7 @@ public:
                 return cudaGetLastError();
             }
         }
-        k_phase1<P, Q, R><<<grid1_, kPhase1Threads, win_bytes_, s>>>(a);
+        k_phase1<P, Q, R><<<grid1_, P1Threads<P, Q, R>::value, win_bytes_, s>>>(a);
         count_launch();
         return cudaGetLastError();
     }
@@ -207,6 +228,8 @@ public:
             if (per_sm != 1) return cudaErrorNotSupported;   // TMEM is sized for one CTA per SM
             const int64_t tiles = (b_.N + 127) / 128;
             grid1_ = (int)std::max<int64_t>(1, std::min<int64_t>((tiles + kTcWG - 1) / kTcWG, num_sms_));
+            args_.win_r0 = window_r0(t_.Nk, kWin);
+            args_.use_win = t_.Nk >= kWin;
             tc_mode_ = mode;
             return cudaSuccess;
         } else {
@@ -233,7 +256,7 @@ public:
     // its phase-2 blocks (ProjRed shapes), whichever is larger
     size_t fused_smem() const
     {
-        const size_t red = ProjRed<P, Q, R>::value ? (size_t)(kPhase1Threads / 32) * ProjRed<P, Q, R>::warp_elems * sizeof(R) : 0;
+        const size_t red = ProjRed<P, Q, R>::value ? (size_t)(P1Threads<P, Q, R>::value / 32) * ProjRed<P, Q, R>::warp_elems * sizeof(R) : 0;
         return std::max(win_bytes_, red);
     }
 
@@ -257,7 +280,7 @@ public:
         a1.tilectr = b_.qcount + 4 + (int)(n % kQSlots);
         a2.out_step = out_prev ? 1 : 0;
         a2.out_next = out_n ? 1 : 0;
-        k_step<P, Q, R><<<grid2f_ + grid1_, kPhase1Threads, fused_smem(), s>>>(a1, a2, grid2f_);
+        k_step<P, Q, R><<<grid2f_ + grid1_, P1Threads<P, Q, R>::value, fused_smem(), s>>>(a1, a2, grid2f_);
         count_launch();
         return cudaGetLastError();
         }
