@@ -254,6 +254,32 @@ __device__ __forceinline__ R knorm2(R kx, R ky)
     else return __fmaf_rn(kx, kx, __fmul_rn(ky, ky));
 }
 
+// Maxima of three: `max3` drops NaN as fmaxf does, `max3_nan` keeps it.  A particle with a NaN node value
+// must not be taken for one inside the window (its cell codes are garbage), while the screen's
+// maximum drops NaN: both maxima over pairs of nodes cost what one over single nodes does.
+__device__ __forceinline__ float max3(float a, float b, float c)
+{
+    float r;
+    asm("max.f32 %0, %1, %2, %3;" : "=f"(r) : "f"(a), "f"(b), "f"(c));
+    return r;
+}
+__device__ __forceinline__ float max3_nan(float a, float b, float c)
+{
+    float r;
+    asm("max.NaN.f32 %0, %1, %2, %3;" : "=f"(r) : "f"(a), "f"(b), "f"(c));
+    return r;
+}
+// max over the nodes of kk, taken in node order
+struct KkMax {
+    float m = 0.0f, n = 0.0f, prev = 0.0f;   // without and with NaN; the even node of a pair
+    __device__ __forceinline__ void add(int q, int Q, float kk)
+    {
+        if (q & 1) { m = max3(m, prev, kk); n = max3_nan(n, prev, kk); }
+        else if (q == Q - 1) { m = fmaxf(m, kk); n = max3_nan(n, kk, kk); }
+        else prev = kk;
+    }
+};
+
 template <int P, int Q, typename R>
 __device__ __forceinline__ bool screen_maybe(const Phys<R> &ph, const Nodes<P, Q, R> &nd, R kkmax, uint32_t xi_bits)
 {
@@ -656,23 +682,27 @@ __device__ __forceinline__ void phase1_pass(const Phys<R> &ph, const Nodes<P, Q,
             // reconstruction, cells and the bound on the majorant
             uint32_t cell[Q];   // FP32: window_code; FP64: (row << 16) | column, ~0 outside the grid
             R kkmax = (R)0;
+            KkMax km;
             F2 inv2, magic2;
             if constexpr (sizeof(R) == 4) { inv2 = f2_pack(ph.inv_dk, ph.inv_dk); magic2 = window_magic(win_r0); }
             recon_all(nd, cx[e], cy[e], [&](int q, R kx, R ky) {
                 if constexpr (sizeof(R) == 4) {
                     cell[q] = window_code<W>(kx, ky, nd.lk2[q], inv2, magic2);
+                    km.add(q, Q, knorm2(kx, ky));
                 } else {
                     int r, l;
                     cell[q] = cell_rl(ph, nd.lkx[q], kx, ky, r, l) ? (uint32_t)((r << 16) | l) : ~0u;
+                    kkmax = fmax(kkmax, knorm2(kx, ky));
                 }
-                kkmax = fmax(kkmax, knorm2(kx, ky));
             });
+            if constexpr (sizeof(R) == 4) kkmax = km.m;
+            const bool in_window = km.n <= kk_in;   // (false for NaN)
             const U4 r = philox4x32_10((uint32_t)i, t.stream_id, t.step, 0u, t.key0, t.key1);
             maybe = screen_maybe(ph, nd, kkmax, r.x);
             if (!maybe) {
                 finished[e] = true;
                 if constexpr (sizeof(R) == 4) {
-                    if (kkmax <= kk_in) {   // every node value lies in the window
+                    if (in_window) {   // every node value lies in the window
 #pragma unroll (kUnrollQ ? Q : 1)
                         for (int q = 0; q < Q; ++q)
                             atomicAdd(reinterpret_cast<uint32_t *>(reinterpret_cast<char *>(swin + (q >> 1) * (W * W)) + (cell[q] & 0xfffcu)),

@@ -89,3 +89,36 @@ def test_batched_histogram_equals_count_of_the_state(shape, Nk, Lk):
     for s, p in zip(b.sims, cases):
         _check(s, p)
     b.close()
+
+
+@pytest.mark.parametrize("precision", ["fp32", "fp64"])
+@pytest.mark.parametrize("shape", ["1x1", "6x6", "21x36", "21x21"])
+def test_non_finite_and_huge_states_leave_the_others_alone(shape, precision):
+    """NaN, infinite and huge coefficients (an uploaded state may hold any): every count of the finite
+    particles is as without them, and a bad particle is counted at most once per node."""
+    from paper_2404_19602_gb300 import build, pgc
+
+    build.build()
+    base, kw = BASE[shape]
+    N = 700
+    p = W.scaled(base, N=N, precision=precision, mech_mask=0, seed=3, **kw)
+    sim = pgc.Simulation(p, max_outputs=4)
+    good = sim.state()
+    sim.close()
+    far = good.copy()
+    bad = np.arange(5, N, 61)
+    far[:, :, bad] = 0.0
+    far[0, 0, bad] = 1e3          # outside the grid, finite
+    vals = [np.nan, np.inf, -np.inf, 1e30, -1e30, 3e38, -6.3e6, 6.3e6]
+    ugly = far.copy()
+    for j, i in enumerate(bad):
+        ugly[j % 2, j % good.shape[1], i] = vals[j % len(vals)]
+    hists = []
+    for state in (far, ugly):
+        s = pgc.Simulation(p, init_khat=good, max_outputs=4)
+        s.set_state(state)
+        s.step(1, 0)
+        hists.append(s.hist()[0].astype(np.int64))
+        s.close()
+    extra = hists[1] - hists[0]
+    assert extra.min() >= 0 and (extra.sum(axis=(1, 2)) <= len(bad)).all()
