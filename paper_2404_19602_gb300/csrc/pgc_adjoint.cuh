@@ -354,7 +354,7 @@ __device__ __forceinline__ void replay_events(const Phys<R> &ph, const Nodes<P, 
                 }
                 if (l == 6) continue;
                 R nkx, nky;
-                final_state(ph, l, kx[s], ky[s], nd.eps0[q], ang, &nkx, &nky);
+                final_state<8>(ph, l, kx[s], ky[s], nd.eps0[q], ang, &nkx, &nky);
                 bool accept = true;
                 if (ph.pauli_mode != 2) {
                     const int cl = cell_of(ph, nd.lkx[q], nkx + nd.dq[q], nky);
@@ -384,7 +384,7 @@ __device__ __forceinline__ void replay_events(const Phys<R> &ph, const Nodes<P, 
             }
             if (l == 6) continue;
             R nkx, nky;
-            final_state(ph, l, kx[s], ky[s], nd.eps0[q], ang, &nkx, &nky);
+            final_state<8>(ph, l, kx[s], ky[s], nd.eps0[q], ang, &nkx, &nky);
             bool accept = true;
             if (ph.pauli_mode != 2) {
                 const int cl = cell_of(ph, nd.lkx[q], nkx + nd.dq[q], nky);

@@ -94,6 +94,19 @@ template <typename R> __device__ __forceinline__ R rfloor(R x);
 template <> __device__ __forceinline__ float rfloor<float>(float x) { return floorf(x); }
 template <> __device__ __forceinline__ double rfloor<double>(double x) { return floor(x); }
 
+// a*b + c*d and a*b - c*d with the contraction written out (the first product fused, the second rounded):
+// left to the compiler, which product it fuses depends on the surrounding code, and kernels that must
+// take the same trajectory bit for bit (two-launch, fused, batched, replayed steps) would differ.
+__device__ __forceinline__ float sum2(float a, float b, float c, float d) { return __fmaf_rn(a, b, __fmul_rn(c, d)); }
+__device__ __forceinline__ double sum2(double a, double b, double c, double d) { return __fma_rn(a, b, __dmul_rn(c, d)); }
+__device__ __forceinline__ float diff2(float a, float b, float c, float d) { return __fmaf_rn(a, b, -__fmul_rn(c, d)); }
+__device__ __forceinline__ double diff2(double a, double b, double c, double d) { return __fma_rn(a, b, -__dmul_rn(c, d)); }
+
+__device__ __forceinline__ float mul_rn(float a, float b) { return __fmul_rn(a, b); }
+__device__ __forceinline__ double mul_rn(double a, double b) { return __dmul_rn(a, b); }
+__device__ __forceinline__ float fma_rn(float a, float b, float c) { return __fmaf_rn(a, b, c); }
+__device__ __forceinline__ double fma_rn(double a, double b, double c) { return __fma_rn(a, b, c); }
+
 // ------------------------------------------------------------------------------------------
 // Cell of a wave-vector on the fixed grid [-Lk, Lk]^2 (Sec. 3); -1 outside.  The FP64 mode
 // gives the cell of the division (as the definition reads, floor_div_f64); the FP32 mode
@@ -199,8 +212,8 @@ __device__ __forceinline__ R edge_T(const Phys<R> &ph, R beta, R c)
 template <typename R>
 __device__ __forceinline__ R rates6(const Phys<R> &ph, R kx, R ky, R eps0, R g[6])
 {
-    const R kk = kx * kx + ky * ky;
-    const R eps = rsqrt_<R>(ph.hvF2 * kk + eps0 * eps0);
+    const R kk = sum2(kx, kx, ky, ky);
+    const R eps = rsqrt_<R>(sum2(eps0, eps0, ph.hvF2, kk));
     const uint32_t m = ph.mech;
     g[0] = (m & 1u) ? ph.Cac * eps : (R)0;
     g[1] = ((m & 2u) && (eps - ph.hwO - eps0 > (R)0)) ? ph.COm * (eps - ph.hwO) : (R)0;
@@ -269,23 +282,38 @@ __device__ __noinline__ R solve_angle(R u, R sgn)
 // Edge final angle: absolute angle with density exp(-beta (c - cos th')^2), inverted through
 // the trapezoid CDF on the n_theta grid, linear between grid points.  The total of the CDF is
 // T(beta, c) (edge_T); one pass up to the target's segment.
-template <typename R>
+// The exponentials of UN grid points are formed together: they do not depend on the running sum, and
+// one at a time the loop waits for each one's latency.  UN = 8 in the collider kernels of their own (6
+// nodes, 5e5 particles: 15.0 -> 12.1 us a launch with the merged angle call below), 1 in the fused
+// step kernel, which instruction fetch bounds (there 8 costs 3 % of the whole step).
+template <typename R, int UN>
 __device__ R edge_angle(const Phys<R> &ph, R beta, R c, R u)
 {
     const int n = ph.n_theta;
-    const R target = u * edge_T<R>(ph, beta, c);
+    const R target = mul_rn(u, edge_T<R>(ph, beta, c)), h2 = (R)0.5 * ph.edge_h;
     R C = (R)0;
     R prev = rexp<R>(-beta * (ph.cosj[0] - c) * (ph.cosj[0] - c));
-    for (int j = 1; j <= n; ++j) {
-        const R x = ph.cosj[j] - c;
-        const R g = rexp<R>(-beta * x * x);
-        const R Cn = C + (R)0.5 * ph.edge_h * (prev + g);
-        if (Cn > target || j == n) {
-            const R frac = fmin(fmax((target - C) / (Cn - C), (R)0), (R)1);
-            return ((R)(j - 1) + frac) * ph.edge_h;
+    for (int j = 1; j <= n; j += UN) {
+        R g[UN];
+#pragma unroll
+        for (int e = 0; e < UN; ++e) {
+            const R x = ph.cosj[min(j + e, n)] - c;
+            g[e] = rexp<R>(-beta * x * x);
         }
-        C = Cn;
-        prev = g;
+        bool hit = false;
+        R C0 = (R)0, C1 = (R)1;
+        int j0 = 0;
+#pragma unroll
+        for (int e = 0; e < UN; ++e) {
+            const R Cn = fma_rn(h2, prev + g[e], C);
+            if (!hit && (Cn > target || j + e >= n)) { hit = true; C0 = C; C1 = Cn; j0 = j + e - 1; }
+            C = Cn;
+            prev = g[e];
+        }
+        if (hit) {
+            const R frac = fmin(fmax((target - C0) / (C1 - C0), (R)0), (R)1);
+            return ((R)j0 + frac) * ph.edge_h;
+        }
     }
     return (R)0;
 }
@@ -298,38 +326,33 @@ struct EventAngles {
     bool have_ac, have_k;
     __device__ void reset(R uu) { u = uu; have_ac = have_k = false; }
     __device__ R ac() { if (!have_ac) { th_ac = solve_angle<R>(u, (R)1); have_ac = true; } return th_ac; }
+    // the angle law of mechanism l: acoustic (0) or K phonon (3, 4); one call site, which the lanes of
+    // a warp that need either law run together
+    __device__ R solved(int l)
+    {
+        if (l == 0 ? !have_ac : !have_k) {
+            const R th = solve_angle<R>(u, l == 0 ? (R)1 : (R)-1);
+            if (l == 0) { th_ac = th; have_ac = true; }
+            else { th_k = th; have_k = true; }
+        }
+        return l == 0 ? th_ac : th_k;
+    }
     __device__ R kk() { if (!have_k) { th_k = solve_angle<R>(u, (R)-1); have_k = true; } return th_k; }
 };
 
-// Final state h^l(k) of mechanism l (0..5) at one node (Sec. 3).  Self scattering (l = 6) is
-// handled by the caller.
+// Final state of a phonon mechanism l (0..4) with the angle's sine and cosine given: |k| of the
+// mechanism, rotated.
 template <typename R>
-__device__ __forceinline__ void final_state(const Phys<R> &ph, int l, R kx, R ky, R eps0,
-                                            EventAngles<R> &ang, R *nkx, R *nky)
+__device__ __forceinline__ void rotate_state(const Phys<R> &ph, int l, R kx, R ky, R kk, R km, R eps0, R st, R ct, R *nkx, R *nky)
 {
-    const R kk = kx * kx + ky * ky;
-    const R km = rsqrt_<R>(kk);
-    if (l == 5) {  // edge: absolute final angle, |k'| = |k|
-        const R c = (km > (R)0) ? kx / km : (R)1;
-        const R th = edge_angle<R>(ph, ph.two_a2 * kk, c, ang.u);
-        R s, co;
-        rsincos<R>(th, &s, &co);
-        *nkx = km * co;
-        *nky = km * s;
-        return;
-    }
     const R ci = (km > (R)0) ? kx / km : (R)1;
     const R si = (km > (R)0) ? ky / km : (R)0;
-    R th, kn;
-    if (l == 0) {
-        th = ang.ac();
-        kn = km;
-    } else {
+    R kn = km;
+    if (l > 0) {
         const bool emit = (l == 1 || l == 3);
         const bool opt = (l == 1 || l == 2);
-        th = opt ? (R)(2.0 * kPi) * ang.u : ang.kk();
-        const R hw = opt ? ph.hwO : ph.hwK;
         if (ph.final_state == 1) {
+            const R hw = opt ? ph.hwO : ph.hwK;
             const R eps = rsqrt_<R>(ph.hvF2 * kk + eps0 * eps0);
             const R ep = emit ? eps - hw : eps + hw;
             kn = rsqrt_<R>(ep * ep - eps0 * eps0) / ph.hvF;
@@ -338,10 +361,39 @@ __device__ __forceinline__ void final_state(const Phys<R> &ph, int l, R kx, R ky
             kn = emit ? km - dk : km + dk;
         }
     }
+    *nkx = kn * diff2(ct, ci, st, si);
+    *nky = kn * sum2(st, ci, ct, si);
+}
+
+// Edge scattering: absolute final angle, |k'| = |k|.
+template <int UN, typename R>
+__device__ __forceinline__ void edge_state(const Phys<R> &ph, R kx, R kk, R km, R u, R *nkx, R *nky)
+{
+    const R c = (km > (R)0) ? kx / km : (R)1;
+    const R th = edge_angle<R, UN>(ph, ph.two_a2 * kk, c, u);
+    R s, co;
+    rsincos<R>(th, &s, &co);
+    *nkx = km * co;
+    *nky = km * s;
+}
+
+// Final state h^l(k) of mechanism l (0..5) at one node (Sec. 3).  Self scattering (l = 6) is
+// handled by the caller.
+template <int UN, typename R>
+__device__ __forceinline__ void final_state(const Phys<R> &ph, int l, R kx, R ky, R eps0,
+                                            EventAngles<R> &ang, R *nkx, R *nky)
+{
+    const R kk = sum2(kx, kx, ky, ky);
+    const R km = rsqrt_<R>(kk);
+    if (l == 5) {
+        edge_state<UN>(ph, kx, kk, km, ang.u, nkx, nky);
+        return;
+    }
+    const bool opt = (l == 1 || l == 2);
+    const R th = opt ? (R)(2.0 * kPi) * ang.u : ang.solved(l);
     R st, ct;
     rsincos<R>(th, &st, &ct);
-    *nkx = kn * (ct * ci - st * si);
-    *nky = kn * (st * ci + ct * si);
+    rotate_state(ph, l, kx, ky, kk, km, eps0, st, ct, nkx, nky);
 }
 
 // Pauli acceptance of a candidate in a cell: f = H / Nmax < eta with eta = m 2^-24 (m odd),

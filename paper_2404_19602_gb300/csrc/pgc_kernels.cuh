@@ -1209,7 +1209,7 @@ __device__ __forceinline__ void collide_particle(const Phys<R> &ph, const Nodes<
                 }
                 if (l == 6) continue;  // self scattering: h^7 = identity
                 R nkx, nky;
-                final_state(ph, l, slot_get(kx, s), slot_get(ky, s), nd.eps0[q], ang, &nkx, &nky);
+                final_state<EXT ? 1 : 8>(ph, l, slot_get(kx, s), slot_get(ky, s), nd.eps0[q], ang, &nkx, &nky);
                 bool accept = true;
                 if (ph.pauli_mode != 2) {
                     const int cl = cell_of(ph, nd.lkx[q], nkx + nd.dq[q], nky);
@@ -1237,7 +1237,7 @@ __device__ __forceinline__ void collide_particle(const Phys<R> &ph, const Nodes<
             }
             if (l == 6) continue;  // self scattering: h^7 = identity
             R nkx, nky;
-            final_state(ph, l, kx[s], ky[s], nd.eps0[q], ang, &nkx, &nky);
+            final_state<EXT ? 1 : 8>(ph, l, kx[s], ky[s], nd.eps0[q], ang, &nkx, &nky);
             bool accept = true;
             if (ph.pauli_mode != 2) {
                 const int cl = cell_of(ph, nd.lkx[q], nkx + nd.dq[q], nky);
