@@ -427,10 +427,9 @@ k_adj_collide(const __grid_constant__ AdjArgs<P, Q, R> a)
     const int lane = threadIdx.x & 31;
     const int r = lane % G;
     const unsigned gmask = (G == 32) ? 0xffffffffu : (((1u << G) - 1u) << (lane - r));
-    const uint32_t gid = (blockIdx.x * blockDim.x + threadIdx.x) / G;
-    const uint32_t ngroups = gridDim.x * blockDim.x / G;
+    const QueueShare qs = queue_share<G>(count, blockIdx.x, gridDim.x);
     double g[NTH] = {0.0, 0.0, 0.0, 0.0};
-    for (uint32_t j = gid; j < count; j += ngroups) {
+    for (uint32_t j = qs.first; j < count; j += qs.stride) {
         const int64_t i = a.queue[j];
         R lx[P], ly[P];
 #pragma unroll

@@ -552,7 +552,7 @@ struct Layout {
     size_t state = 0, hist = 0, scratch = 0;
     size_t off_queue = 0, off_qcount = 0, off_counters = 0, off_nmax = 0, off_part1 = 0, off_part2 = 0,
            off_partN = 0, off_marks = 0, off_tables = 0, off_series = 0, off_recon = 0, off_tmpmax = 0,
-           off_obs = 0, off_colsum = 0, off_fdtab = 0;
+           off_obs = 0, off_colsum = 0, off_fdtab = 0, off_edgetab = 0;
     int rec_len = 0;
 };
 }  // namespace
@@ -623,6 +623,7 @@ static pgc_status check_config(const pgc_config *c, Layout *L, std::string *msg)
     L->off_obs = take((size_t)(kObsGrid * kObsZ * 3 + kObsZ * 4) * 8);
     L->off_colsum = take((size_t)64 * 3 * 8);
     L->off_fdtab = take(kFdTableBytes);
+    L->off_edgetab = take(c->precision == PGC_FP64 ? (size_t)(c->n_theta_edge + 1) * kEdgeK * 8 : 0);
     L->scratch = off;
     return PGC_OK;
 }
@@ -749,6 +750,7 @@ pgc_status pgc_init(const pgc_config *cfg, void *d_state, void *d_hist, void *d_
     b.mark_words = L.mark_words;
     b.tables = scr + L.off_tables;
     b.fdtab = (double *)(scr + L.off_fdtab);
+    if (cfg->precision == PGC_FP64) b.edge_tab = (double *)(scr + L.off_edgetab);
     b.recon_hist = (uint32_t *)(scr + L.off_recon);
     b.key0 = (uint32_t)cfg->seed;
     b.key1 = (uint32_t)(cfg->seed >> 32);

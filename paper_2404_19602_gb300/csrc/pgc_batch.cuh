@@ -169,9 +169,8 @@ k_phase2_batch(const __grid_constant__ BatchArgs<P, Q, R> a)
     const int lane = threadIdx.x & 31;
     const int r = lane % G;
     const unsigned gmask = (G == 32) ? 0xffffffffu : (((1u << G) - 1u) << (lane - r));
-    const uint32_t gid = (blockIdx.x * blockDim.x + threadIdx.x) / G;
-    const uint32_t ngroups = gridDim.x * blockDim.x / G;
-    for (uint32_t j = gid; j < count; j += ngroups) {
+    const QueueShare qs = queue_share<G>(count, blockIdx.x, gridDim.x);
+    for (uint32_t j = qs.first; j < count; j += qs.stride) {
         const int64_t g = a.queue[j];
         const int c = find_case(sbase, a.ncases + 1, g);
         const CaseDev<P, Q, R> &cd = a.cases[c];

@@ -12,6 +12,7 @@ namespace pgc {
 
 constexpr int kMaxTheta = 256;   // upper bound of the edge trapezoid points
 constexpr int kSerMax = 17;      // maximum order + 1 of the edge-integral series
+constexpr int kEdgeK = 26;       // powers per row of Phys::edge_tab (even: rows of double2)
 constexpr double kPi = 3.14159265358979323846;
 
 // ------------------------------------------------------------------------------------------
@@ -37,6 +38,7 @@ struct Phys {
     // power series of T in beta (see edge_T): coefficient (j, m) of beta^j (c^2)^(j-m)
     R tser[kSerMax * kSerMax];
     R beta_ser;           // the series is used for beta <= beta_ser
+    const double *edge_tab;  // FP64: prefix sums of cos^k over the trapezoid grid (edge_angle), or nullptr
     int32_t J;            // series order
     uint32_t mech;
     int32_t n_theta;
@@ -183,6 +185,20 @@ __device__ __forceinline__ int cell_of(const Phys<R> &ph, R lkx, R kx, R ky)
 template <typename R>
 __device__ __forceinline__ R edge_T(const Phys<R> &ph, R beta, R c)
 {
+    if (sizeof(R) == 8 && beta <= (R)0.02 && beta <= ph.beta_ser) {
+        // FP64, the |k| <= 1 nm^-1 most states have: nine terms reach rounding, (4 beta)^10 / 10! < 1e-17
+        const R x = c * c;
+        R acc = (R)0;
+#pragma unroll
+        for (int j = 9; j >= 0; --j) {
+            const R *a = &ph.tser[j * kSerMax];
+            R p = a[0];
+#pragma unroll
+            for (int m = 1; m <= j; ++m) p = p * x + a[m];
+            acc = acc * beta + p;
+        }
+        return (R)(2.0 * kPi) * acc;
+    }
     if (beta <= ph.beta_ser) {
         constexpr int J = (sizeof(R) == 8) ? 16 : 10;
         const R x = c * c;
@@ -256,10 +272,12 @@ __device__ __noinline__ R solve_angle(R u, R sgn)
 {
     // f(th) = th + sgn sin th - 2 pi u is non-decreasing on [0, 2pi]; safeguarded Newton from a
     // start that captures the cubic behaviour at the stationary point (th = pi for sgn = +1,
-    // th = 0 or 2pi for sgn = -1).
+    // th = 0 or 2pi for sgn = -1).  FP64 starts from the FP32 root: two or three iterations of its slow
+    // sincos instead of six or seven.
     const R twopi = (R)(2.0 * kPi), t = twopi * u;
     R lo = (R)0, hi = twopi, th;
-    if (sgn > (R)0) th = (R)kPi + cbrt((R)6 * (t - (R)kPi));
+    if constexpr (sizeof(R) == 8) th = (R)solve_angle<float>((float)u, (float)sgn);   // (u has 24 bits)
+    else if (sgn > (R)0) th = (R)kPi + cbrt((R)6 * (t - (R)kPi));
     else th = (t < (R)kPi) ? cbrt((R)6 * t) : twopi - cbrt((R)6 * (twopi - t));
     th = fmin(fmax(th, (R)0), twopi);
     const int iters = (sizeof(R) == 8) ? 60 : 30;
@@ -279,6 +297,52 @@ __device__ __noinline__ R solve_angle(R u, R sgn)
     return th;
 }
 
+// The FP64 edge angle without the exponentials: exp(-beta (x - c)^2) = exp(-beta c^2) sum_k h_k x^k with
+// the Hermite recurrence (k + 1) h_{k+1} = 2 beta (c h_k - h_{k-1}), so the trapezoid CDF at grid point j is
+// h exp(-beta c^2) sum_k h_k S_k[j] with the prefix sums S_k[j] of cos^k (edge_tab).  The segment of the
+// target is found by interpolation in the CDF (nearly linear: beta is small), three or four points.
+// The FP64 pipe issues one warp instruction per 16 clocks, and 64 exponentials in turn were 15 us of a
+// chain.  17 powers reach 1e-17 for beta <= 0.02, 26 for beta <= 0.25.
+__device__ inline double edge_angle_tab(const Phys<double> &ph, double beta, double c, double u)
+{
+    const int n = ph.n_theta;
+    const bool small = beta <= 0.02;
+    constexpr int K0 = 18;
+    double h[kEdgeK];
+    const double b2 = 2.0 * beta, bc = b2 * c;
+    h[0] = 1.0;
+    h[1] = bc;
+#pragma unroll
+    for (int k = 1; k < K0 - 1; ++k) h[k + 1] = (bc * h[k] - b2 * h[k - 1]) * (1.0 / (k + 1));
+    if (!small) {
+#pragma unroll
+        for (int k = K0 - 1; k < kEdgeK - 1; ++k) h[k + 1] = (bc * h[k] - b2 * h[k - 1]) * (1.0 / (k + 1));
+    }
+    auto cdf = [&](int j) {
+        const double2 *row = reinterpret_cast<const double2 *>(ph.edge_tab + (size_t)j * kEdgeK);
+        double s0 = 0.0, s1 = 0.0;
+#pragma unroll
+        for (int k = 0; k < K0; k += 2) { const double2 v = row[k / 2]; s0 += h[k] * v.x; s1 += h[k + 1] * v.y; }
+        if (!small) {
+#pragma unroll
+            for (int k = K0; k < kEdgeK; k += 2) { const double2 v = row[k / 2]; s0 += h[k] * v.x; s1 += h[k + 1] * v.y; }
+        }
+        return s0 + s1;
+    };
+    // total and target in units of h exp(-beta c^2); the total's value at n closes the bracket
+    const double total = edge_T<double>(ph, beta, c) * exp(beta * c * c) / ph.edge_h, target = u * total;
+    int lo = 0, hi = n;
+    double Dlo = 0.0, Dhi = total;
+    while (hi - lo > 1) {
+        int m = lo + (int)((target - Dlo) / (Dhi - Dlo) * (hi - lo));
+        m = min(max(m, lo + 1), hi - 1);
+        const double D = cdf(m);
+        if (D > target) { hi = m; Dhi = D; } else { lo = m; Dlo = D; }
+    }
+    const double frac = fmin(fmax((target - Dlo) / (Dhi - Dlo), 0.0), 1.0);
+    return ((double)lo + frac) * ph.edge_h;
+}
+
 // Edge final angle: absolute angle with density exp(-beta (c - cos th')^2), inverted through
 // the trapezoid CDF on the n_theta grid, linear between grid points.  The total of the CDF is
 // T(beta, c) (edge_T); one pass up to the target's segment.
@@ -289,6 +353,9 @@ __device__ __noinline__ R solve_angle(R u, R sgn)
 template <typename R, int UN>
 __device__ R edge_angle(const Phys<R> &ph, R beta, R c, R u)
 {
+    if constexpr (sizeof(R) == 8) {
+        if (ph.edge_tab && beta <= (R)0.25) return edge_angle_tab(ph, beta, c, u);
+    }
     const int n = ph.n_theta;
     const R target = mul_rn(u, edge_T<R>(ph, beta, c)), h2 = (R)0.5 * ph.edge_h;
     R C = (R)0;

@@ -59,6 +59,7 @@ struct DevBuffers {
     int64_t mark_words = 0;
     void *tables = nullptr;         // device copy of the node tables (kTableBytes) or nullptr
     double *fdtab = nullptr;        // table of the Fermi-Dirac inverse (pgc_fd.cuh) or nullptr
+    double *edge_tab = nullptr;     // prefix sums of the FP64 edge angle (Phys::edge_tab) or nullptr
     uint32_t *recon_hist = nullptr; // [Nk*Nk]
     uint32_t key0 = 0, key1 = 0, stream_id = 0;
 };

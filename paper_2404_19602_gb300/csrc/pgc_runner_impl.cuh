@@ -6,6 +6,7 @@
 #include <algorithm>
 #include <cmath>
 #include <cstring>
+#include <vector>
 
 #include "pgc_kernels.cuh"
 #include "pgc_kernels_tc.cuh"
@@ -289,6 +290,21 @@ public:
     cudaError_t upload_tables(cudaStream_t s) override
     {
         if (!b_.tables) return cudaSuccess;
+        if (args_.ph.edge_tab) {   // prefix sums of cos^k with the trapezoid's half weights at both ends
+            const int n = t_.n_theta;
+            std::vector<double> run(kEdgeK, 0.0);
+            std::vector<double> &tab = edge_host_;   // lives as long as the copy may
+            tab.assign((size_t)(n + 1) * kEdgeK, 0.0);
+            for (int j = 0; j <= n; ++j) {
+                double x = std::cos(2.0 * kPi * j / n), xk = 1.0;
+                for (int k = 0; k < kEdgeK; ++k, xk *= x) {
+                    run[k] += xk;
+                    tab[(size_t)j * kEdgeK + k] = run[k] - 0.5 * (1.0 + xk);
+                }
+            }
+            cudaError_t e = cudaMemcpyAsync(b_.edge_tab, tab.data(), tab.size() * 8, cudaMemcpyHostToDevice, s);
+            if (e != cudaSuccess) return e;
+        }
         return cudaMemcpyAsync(b_.tables, &args_.nd, sizeof(Nodes<P, Q, R>), cudaMemcpyHostToDevice, s);
     }
 
@@ -372,6 +388,7 @@ private:
             for (int m = 0; m < kSerMax; ++m)
                 p.tser[j * kSerMax + m] = (R)((m <= j) ? ((j & 1) ? -1.0 : 1.0) / fact * binom(2 * j, 2 * m) * binom(2 * m, m) / std::pow(4.0, m) : 0.0);
         }
+        p.edge_tab = (sizeof(R) == 8 && t.n_theta >= 32) ? b_.edge_tab : nullptr;
         p.mech = t.mech;
         p.n_theta = t.n_theta;
         p.pauli_mode = t.pauli_mode;
@@ -384,6 +401,7 @@ private:
     DevBuffers b_;
     StepArgs<P, Q, R> args_{};
     InitArgs<P, Q> init_{};
+    std::vector<double> edge_host_;
     int grid1_ = 1;
     size_t win_bytes_ = 0;
     int grid2_ = 1;
