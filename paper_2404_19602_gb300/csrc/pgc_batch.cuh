@@ -55,7 +55,7 @@ struct BatchArgs {
     uint32_t *done;            // phase-2 block completion counter
     int32_t moments_every;
     int32_t win_r0, use_win;
-    R kk_in;                   // as in StepArgs, common to the cases (the batched kernels run the Lie splitting)
+    float kk_in;                   // as in StepArgs, common to the cases (the batched kernels run the Lie splitting)
     int32_t rec_len;
     double vF_ms;
 };
@@ -83,7 +83,7 @@ k_phase1_batch(const __grid_constant__ BatchArgs<P, Q, R> a)
     __shared__ typename MomAcc<R>::T smom[NW][Q * 3];
     __shared__ int64_t stile[kBatchMaxCases + 1];
     __shared__ __align__(16) uint32_t snd[(sizeof(Nodes<P, Q, R>) + 3) / 4];
-    __shared__ uint32_t s_aside[sizeof(R) == 4 ? NW : 1][sizeof(R) == 4 ? AsideList<PPT>::cap : 1];
+    __shared__ uint32_t s_aside[NW][AsideList<PPT>::cap];
     extern __shared__ __align__(16) uint32_t swin[];
     const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
     const int64_t step = *a.d_step;
@@ -95,7 +95,7 @@ k_phase1_batch(const __grid_constant__ BatchArgs<P, Q, R> a)
     const int64_t NN = (int64_t)a.ph.Nk * a.ph.Nk;
     const int64_t helems = (int64_t)Q * NN;
     int cur = -1, n_aside = 0;
-    uint32_t *aside = s_aside[sizeof(R) == 4 ? warp : 0];
+    uint32_t *aside = s_aside[warp];
     unsigned int oog = 0u;
     for (int64_t tile = blockIdx.x; tile < a.ntiles; tile += gridDim.x) {
         const int c = find_case(stile, a.ncases + 1, tile);
@@ -131,7 +131,7 @@ k_phase1_batch(const __grid_constant__ BatchArgs<P, Q, R> a)
         for (int64_t base = p0; base < p1; base += (int64_t)blockDim.x * PPT)
             phase1_pass<P, Q, R, HistWin<P, Q, R>::batchW, PPT>(a.ph, nd, t, base + (int64_t)threadIdx.x * PPT, swin, a.win_r0, a.use_win != 0, a.kk_in,
                                       out, smom[warp], aside, n_aside, oog);
-        if (sizeof(R) == 4 && n_aside > 0) {
+        if (n_aside > 0) {
             count_aside<P, Q, R, HistWin<P, Q, R>::batchW>(a.ph, nd, t, aside, n_aside, swin, a.win_r0, a.use_win != 0, oog);
             n_aside = 0;
         }
@@ -335,7 +335,7 @@ public:
         constexpr int W = HistWin<P, Q, R>::batchW;
         a_.use_win = t0.Nk >= W;
         a_.win_r0 = window_r0(t0.Nk, W);
-        a_.kk_in = a_.use_win ? (R)window_kk(t0, W) : (R)-1;
+        a_.kk_in = a_.use_win ? (float)window_kk(t0, W) : -1.0f;
         a_.rec_len = 1 + 4 * Q + 8;
         a_.vF_ms = t0.vF_ms;
         win_bytes_ = a_.use_win ? HistWin<P, Q, R>::batch_bytes : 0;

@@ -19,6 +19,12 @@ constexpr double kPi = 3.14159265358979323846;
 // Physical constants of one context, prepared on the host in FP64 and stored in R.
 // Rates are in 1/fs; energies eV; wave-vectors nm^-1.
 // ------------------------------------------------------------------------------------------
+// FP32 copies of what the streaming screen of the FP64 mode needs (see screen_f32).
+struct ScreenF {
+    float hvF2, inv_dk, alpha1, dt, Cac, COm, COp, CKm, CKp, hwO, hwK, Cedg, bound_edge, Csum;
+    uint32_t mech;
+};
+
 template <typename R>
 struct Phys {
     R hvF, hvF2;          // hbar vF (eV nm) and its square
@@ -46,6 +52,7 @@ struct Phys {
     int32_t final_state;  // 0 paper, 1 exact energy
     int32_t max_coll;
     int32_t Nk;
+    ScreenF f;            // FP64 mode
 };
 
 // ------------------------------------------------------------------------------------------
@@ -248,8 +255,8 @@ __device__ __forceinline__ R rates6(const Phys<R> &ph, R kx, R ky, R eps0, R g[6
 
 // Upper bound of sum_nu Gamma_nu over all states with energy <= eps and band minimum <= eps0max:
 // every closed form is non-decreasing in eps, the Heaviside factors are dropped, T <= 2pi.
-template <typename R>
-__device__ __forceinline__ R rate_bound(const Phys<R> &ph, R eps, R eps0max)
+template <typename R, typename PH>
+__device__ __forceinline__ R rate_bound(const PH &ph, R eps, R eps0max)
 {
     const uint32_t m = ph.mech;
     R s = (R)0;

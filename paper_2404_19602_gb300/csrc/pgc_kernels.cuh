@@ -97,7 +97,7 @@ struct Nodes {
     unsigned long long psi2[(TensorShape<P, Q>::value || sizeof(R) == 8) ? 1 : Q * P];
     unsigned long long wpsi2[(TensorShape<P, Q>::value || sizeof(R) == 8) ? 1 : Q * P];
     unsigned long long a1_2[36], b2_2[36];
-    unsigned long long lk2[sizeof(R) == 8 ? 1 : Q];   // FP32: (lkx[q], Lk)
+    unsigned long long lk2[Q];   // (lkx[q], Lk) in FP32
 };
 
 template <int P, int Q, typename R>
@@ -123,7 +123,7 @@ struct StepArgs {
     int32_t out_step;        // 1: accumulate the moments of the post-step state
     int32_t win_r0;          // first row / column of the shared-memory window
     int32_t use_win;         // 1: phase 1 counts into the shared-memory window
-    R kk_in;                 // |k|^2 up to which a node value's cell lies in the window (< 0: none known to)
+    float kk_in;             // |k|^2 up to which a node value's cell lies in the window (< 0: none known to)
     // collider bitmaps (bit i of word i / 32), all optional (nullptr)
     const uint32_t *skip;    // phase 1: particles queued at step n - 1, owned by a concurrent phase 2
     uint32_t *mark;          // phase 1: set for every particle queued at step n
@@ -289,6 +289,19 @@ __device__ __forceinline__ bool screen_maybe(const Phys<R> &ph, const Nodes<P, Q
     return lnxi < gub * ph.dt;
 }
 
+// The FP64 screen decided in FP32 where the two cannot differ: 1 collides or may, 0 does not, -1
+// undecided (to be taken in FP64).  kkmax, the energy, each rate and the logarithm carry a few FP32
+// roundings; 3e-5 of the bound plus 2e-6 of all rate prefactors times the energy (the emission terms
+// subtract the phonon energy) is more than ten times their sum, and the undecided share is ~1e-6.
+__device__ __forceinline__ int screen_f32(const ScreenF &f, float kkmax, float eps0_max, uint32_t xi_bits)
+{
+    const float lnxi = -logf(u01<float>(xi_bits));
+    const float emax = sqrtf(f.hvF2 * kkmax + eps0_max * eps0_max);
+    const float x = f.alpha1 * rate_bound(f, emax, eps0_max) * 1.0001f * f.dt;
+    const float tol = 3e-5f * x + 2e-6f * f.Csum * emax;
+    return lnxi > x + tol ? 0 : (lnxi < x - tol ? 1 : -1);
+}
+
 template <int P, int Q, typename R>
 __device__ __forceinline__ void load_coeffs(const StepArgs<P, Q, R> &a, int64_t i, R cx[P], R cy[P])
 {
@@ -351,6 +364,23 @@ __device__ __forceinline__ uint32_t window_code(float kx, float ky, unsigned lon
 {
     const F2 s = f2_add_rd(f2_mul(f2_add(f2_pack(kx, ky), lk2), inv2), magic2);
     return (uint32_t)s.v * (4u * W) + (uint32_t)(s.v >> 32);
+}
+// The same for the FP64 mode from the node value rounded to FP32, with the distance of the FP32 cell
+// coordinates from the nearest cell edge (in `edge`, the smallest so far): the FP64 cell is the same
+// unless that distance is within the rounding (kCellGuard * Nk cells).
+constexpr float kCellGuard = 1e-6f;   // of Nk: four roundings of 6e-8 Nk, four times over
+template <int W>
+__device__ __forceinline__ uint32_t window_code_f64(double kx, double ky, unsigned long long lk2, F2 inv2, int win_r0, float &edge)
+{
+    const float m = 8388608.0f - (float)win_r0;
+    const F2 y = f2_mul(f2_add(f2_pack((float)kx, (float)ky), lk2), inv2);
+    const F2 s = f2_add_rd(y, f2_pack(m, m));
+    float yx, yy, sx, sy;
+    f2_unpack(y, yx, yy);
+    f2_unpack(s, sx, sy);
+    const float fx = yx - (float)win_r0 - (sx - 8388608.0f), fy = yy - (float)win_r0 - (sy - 8388608.0f);
+    edge = fminf(edge, fminf(fminf(fx, 1.0f - fx), fminf(fy, 1.0f - fy)));
+    return (uint32_t)s.v * (4u * W) + 4u * (uint32_t)(s.v >> 32);
 }
 __device__ __forceinline__ F2 window_magic(int r0) { return f2_pack(8388608.0f - (float)r0, 2097152.0f - (float)r0); }
 
@@ -595,7 +625,7 @@ struct P1Target {
 
 // The particles of a warp with a node value outside the circle of the window (kk_in), put aside in
 // shared memory: a rolled pass over their nodes for one lane costs a warp as much as for 32, so they
-// are taken 32 at a time (FP32 kernels; at most 31 stay between passes).
+// are taken 32 at a time (at most 31 stay between passes).
 template <int PPT> struct AsideList { static constexpr int cap = 32 * (PPT + 1); };
 
 // Counts the histogram cells of n <= 32 such particles (one per lane) from their stored state.
@@ -632,7 +662,7 @@ __device__ __forceinline__ void count_aside(const Phys<R> &ph, const Nodes<P, Q,
 // (PPT particles per thread; i0 a multiple of PPT.)
 template <int P, int Q, typename R, int W = HistWin<P, Q, R>::W, int PPT = Phase1PPT<P>::value>
 __device__ __forceinline__ void phase1_pass(const Phys<R> &ph, const Nodes<P, Q, R> &nd, const P1Target<R> &t,
-                                            int64_t i0, uint32_t *swin, int win_r0, bool use_win, R kk_in, bool out_step,
+                                            int64_t i0, uint32_t *swin, int win_r0, bool use_win, float kk_in, bool out_step,
                                             typename MomAcc<R>::T *smom_warp, uint32_t *aside, int &n_aside,
                                             unsigned int &oog)
 {
@@ -680,51 +710,51 @@ __device__ __forceinline__ void phase1_pass(const Phys<R> &ph, const Nodes<P, Q,
         bool maybe = false, put_aside = false;
         if (any && i < t.N && !((skipbits >> e) & 1u)) {
             // reconstruction, cells and the bound on the majorant
-            uint32_t cell[Q];   // FP32: window_code; FP64: (row << 16) | column, ~0 outside the grid
-            R kkmax = (R)0;
-            KkMax km;
-            F2 inv2, magic2;
-            if constexpr (sizeof(R) == 4) { inv2 = f2_pack(ph.inv_dk, ph.inv_dk); magic2 = window_magic(win_r0); }
-            recon_all(nd, cx[e], cy[e], [&](int q, R kx, R ky) {
-                if constexpr (sizeof(R) == 4) {
+            uint32_t cell[Q];   // window_code
+            const F2 inv2 = sizeof(R) == 4 ? f2_pack((float)ph.inv_dk, (float)ph.inv_dk) : f2_pack(ph.f.inv_dk, ph.f.inv_dk);
+            const U4 r = philox4x32_10((uint32_t)i, t.stream_id, t.step, 0u, t.key0, t.key1);
+            bool in_window;
+            if constexpr (sizeof(R) == 4) {
+                const F2 magic2 = window_magic(win_r0);
+                KkMax km;
+                recon_all(nd, cx[e], cy[e], [&](int q, R kx, R ky) {
                     cell[q] = window_code<W>(kx, ky, nd.lk2[q], inv2, magic2);
                     km.add(q, Q, knorm2(kx, ky));
-                } else {
-                    int r, l;
-                    cell[q] = cell_rl(ph, nd.lkx[q], kx, ky, r, l) ? (uint32_t)((r << 16) | l) : ~0u;
-                    kkmax = fmax(kkmax, knorm2(kx, ky));
+                });
+                in_window = km.n <= kk_in;   // (false for NaN)
+                maybe = screen_maybe(ph, nd, km.m, r.x);
+            } else {
+                // FP64: cells and screen in FP32 where FP32 is certain of them (the FP64 pipe issues one warp
+                // instruction per 16 clocks; the reconstruction is what it has to do), else in FP64
+                KkMax km;
+                float edge = 1.0f;
+                recon_all(nd, cx[e], cy[e], [&](int q, R kx, R ky) {
+                    cell[q] = window_code_f64<W>(kx, ky, nd.lk2[q], inv2, win_r0, edge);
+                    const float xf = (float)kx, yf = (float)ky;
+                    km.add(q, Q, xf * xf + yf * yf);
+                });
+                const int sc = screen_f32(ph.f, km.n, (float)nd.eps0_max, r.x);
+                maybe = sc > 0;
+                if (sc < 0) {
+                    R kk = (R)0;
+                    recon_all_rolled(nd, cx[e], cy[e], [&](int, R kx, R ky) { kk = fmax(kk, knorm2(kx, ky)); });
+                    maybe = screen_maybe(ph, nd, kk, r.x);
                 }
-            });
-            if constexpr (sizeof(R) == 4) kkmax = km.m;
-            const bool in_window = km.n <= kk_in;   // (false for NaN)
-            const U4 r = philox4x32_10((uint32_t)i, t.stream_id, t.step, 0u, t.key0, t.key1);
-            maybe = screen_maybe(ph, nd, kkmax, r.x);
+                in_window = km.n <= kk_in && edge > kCellGuard * (float)ph.Nk;
+            }
             if (!maybe) {
                 finished[e] = true;
-                if constexpr (sizeof(R) == 4) {
-                    if (in_window) {   // every node value lies in the window
+                if (in_window) {   // every node value lies in the window
 #pragma unroll (kUnrollQ ? Q : 1)
-                        for (int q = 0; q < Q; ++q)
-                            atomicAdd(reinterpret_cast<uint32_t *>(reinterpret_cast<char *>(swin + (q >> 1) * (W * W)) + (cell[q] & 0xfffcu)),
-                                      (q & 1) ? 0x10000u : 1u);
-                    } else {
-                        put_aside = true;
-                    }
+                    for (int q = 0; q < Q; ++q)
+                        atomicAdd(reinterpret_cast<uint32_t *>(reinterpret_cast<char *>(swin + (q >> 1) * (W * W)) + (cell[q] & 0xfffcu)),
+                                  (q & 1) ? 0x10000u : 1u);
                 } else {
-#pragma unroll (kUnrollQ ? Q : 1)
-                    for (int q = 0; q < Q; ++q) {
-                        if (cell[q] == ~0u) { ++oog; continue; }
-                        const int r = (int)(cell[q] >> 16), l = (int)(cell[q] & 0xffffu);
-                        const int rr = r - win_r0, ll = l - win_r0;
-                        if (use_win && (unsigned)rr < (unsigned)W && (unsigned)ll < (unsigned)W)
-                            atomicAdd(&swin[(q >> 1) * (W * W) + rr * W + ll], 1u << ((q & 1) << 4));
-                        else
-                            atomicAdd(&t.Hnext[(int64_t)q * NN + r * ph.Nk + l], 1u);
-                    }
+                    put_aside = true;
                 }
             }
         }
-        if constexpr (sizeof(R) == 4) {
+        {
             const unsigned int am = __ballot_sync(0xffffffffu, put_aside);
             if (am) {
                 if (put_aside) aside[n_aside + __popc(am & ((1u << lane) - 1u))] = (uint32_t)i;
@@ -803,11 +833,9 @@ __device__ __forceinline__ void phase1_pass(const Phys<R> &ph, const Nodes<P, Q,
             }
         }
     }
-    if constexpr (sizeof(R) == 4) {
-        while (n_aside >= 32) {
-            n_aside -= 32;
-            count_aside<P, Q, R, W>(ph, nd, t, aside + n_aside, 32, swin, win_r0, use_win, oog);
-        }
+    while (n_aside >= 32) {
+        n_aside -= 32;
+        count_aside<P, Q, R, W>(ph, nd, t, aside + n_aside, 32, swin, win_r0, use_win, oog);
     }
 }
 
@@ -865,9 +893,9 @@ __device__ __forceinline__ void phase1_block(const StepArgs<P, Q, R> &a, int bid
     constexpr int NW = P1Threads<P, Q, R>::value / 32;
     __shared__ typename MomAcc<R>::T smom[NW][Q * 3];
     __shared__ uint32_t s_tile;
-    __shared__ uint32_t s_aside[sizeof(R) == 4 ? NW : 1][sizeof(R) == 4 ? AsideList<PPT>::cap : 1];
+    __shared__ uint32_t s_aside[NW][AsideList<PPT>::cap];
     const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
-    uint32_t *aside = s_aside[sizeof(R) == 4 ? warp : 0];
+    uint32_t *aside = s_aside[warp];
     int n_aside = 0;
     if (a.use_win) clear_window<Q, HistWin<P, Q, R>::W>(swin);
     if (a.out_step)
@@ -933,7 +961,7 @@ __device__ __forceinline__ void phase1_block(const StepArgs<P, Q, R> &a, int bid
                                  a.out_step != 0, smom[warp], aside, n_aside, oog);
         }
     }
-    if (sizeof(R) == 4 && n_aside > 0)
+    if (n_aside > 0)
         count_aside<P, Q, R, HistWin<P, Q, R>::W>(a.ph, a.nd, t, aside, n_aside, swin, a.win_r0, a.use_win != 0, oog);
     oog = warp_sum(oog);
     if (lane == 0 && oog) atomicAdd(&a.counters[4], (unsigned long long)oog);

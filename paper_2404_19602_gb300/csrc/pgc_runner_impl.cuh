@@ -24,7 +24,7 @@ inline double window_kk(const HostTables &t, int W)
     double xs = 0.0;
     for (double x : t.xs) xs = std::max(xs, std::fabs(x));
     const double rad = (std::min(0.5 * t.Nk - r0, r0 + W - 0.5 * t.Nk) - 0.01) * t.dk - xs;
-    return rad > 0.0 ? rad * rad * (1.0 - 1e-6) : -1.0;
+    return rad > 0.0 ? rad * rad * (1.0 - 1e-5) : -1.0;
 }
 
 template <int P, int Q, typename R>
@@ -41,8 +41,8 @@ public:
             nd.dq[q] = (R)t.dq[q];
             nd.lkx[q] = (R)(t.Lk - t.xs[q]);   // Lie: the grid's Lk itself
             nd.xs[q] = (R)t.xs[q];
-            if constexpr (sizeof(R) == 4) {   // (lkx, Lk) as the two-lane operand of window_code
-                const float lo = nd.lkx[q], hi = (float)t.Lk;
+            {   // (lkx, Lk) as the two-lane operand of window_code
+                const float lo = (float)(t.Lk - t.xs[q]), hi = (float)t.Lk;
                 uint32_t ul, uh;
                 std::memcpy(&ul, &lo, 4);
                 std::memcpy(&uh, &hi, 4);
@@ -115,7 +115,7 @@ public:
         grid1_ = (int)std::max<int64_t>(1, std::min<int64_t>({need, (int64_t)num_sms * per_sm, (int64_t)kMaxGrid1}));
         args_.use_win = win ? 1 : 0;
         if (!win) win_bytes_ = 0;
-        args_.kk_in = win ? (R)window_kk(t, W) : (R)-1;
+        args_.kk_in = win ? (float)window_kk(t, W) : -1.0f;
         // phase 2: one resident wave (its work is one latency-bound collision chain per group)
         int per_sm2 = 0;
         cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm2, k_phase2<P, Q, R, true>, kPhase2Threads, 0);
@@ -389,6 +389,15 @@ private:
                 p.tser[j * kSerMax + m] = (R)((m <= j) ? ((j & 1) ? -1.0 : 1.0) / fact * binom(2 * j, 2 * m) * binom(2 * m, m) / std::pow(4.0, m) : 0.0);
         }
         p.edge_tab = (sizeof(R) == 8 && t.n_theta >= 32) ? b_.edge_tab : nullptr;
+        {
+            ScreenF &f = p.f;
+            f.hvF2 = (float)(t.hvF * t.hvF); f.inv_dk = (float)(1.0 / t.dk); f.alpha1 = (float)(1.0 + t.alpha); f.dt = (float)t.dt;
+            f.Cac = (float)t.Cac; f.COm = (float)(t.CO * (t.nO + 1.0)); f.COp = (float)(t.CO * t.nO);
+            f.CKm = (float)(t.CK * (t.nK + 1.0)); f.CKp = (float)(t.CK * t.nK); f.hwO = (float)t.hwO; f.hwK = (float)t.hwK;
+            f.Cedg = (float)t.Cedg; f.bound_edge = (float)(2.0 * kPi * (1.0 + 1e-5));
+            f.Csum = (float)((1.0 + t.alpha) * t.dt * (t.Cac + t.CO * (2.0 * t.nO + 1.0) + t.CK * (2.0 * t.nK + 1.0) + t.Cedg * t.eps0_max * 7.0));
+            f.mech = t.mech;
+        }
         p.mech = t.mech;
         p.n_theta = t.n_theta;
         p.pauli_mode = t.pauli_mode;
