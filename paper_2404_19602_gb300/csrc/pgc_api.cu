@@ -408,44 +408,62 @@ struct ObsFin {
     int nz, g;
 };
 
-__global__ void __launch_bounds__(128)
+// Thread t sums column t % 96 over the rows congruent to t / 96 modulo kObsFinSlots, then the slots in
+// order (one thread per column took 26 us for 304 rows, a chain of FP64 adds; 20 us for 608 now).
+constexpr int kObsFinSlots = 8;
+__global__ void __launch_bounds__(kObsZ * 3 * kObsFinSlots)
 k_obs_fin(const double *part, const __grid_constant__ ObsFin f, double *out)
 {
-    __shared__ double S[kObsZ * 3];
-    const int t = threadIdx.x;
-    if (t < kObsZ * 3) {
+    __shared__ double S[kObsFinSlots][kObsZ * 3];
+    const int t = threadIdx.x, col = t % (kObsZ * 3), slot = t / (kObsZ * 3);
+    S[slot][col] = strided_sum(part, slot, f.g, kObsFinSlots, kObsZ * 3, col, 0.0);
+    __syncthreads();
+    if (slot == 0) {
         double s = 0.0;
-        s = strided_sum(part, 0, f.g, 1, kObsZ * 3, t, s);
-        S[t] = s;
+#pragma unroll
+        for (int k = 0; k < kObsFinSlots; ++k) s += S[k][col];
+        S[0][col] = s;
     }
     __syncthreads();
     if (t < f.nz) {
         const double qe = 1.602176634e-19;
-        const double vx = S[t * 3 + 0] * f.scale_v, vy = S[t * 3 + 1] * f.scale_v;
+        const double vx = S[0][t * 3 + 0] * f.scale_v, vy = S[0][t * 3 + 1] * f.scale_v;
         out[t * 4 + 0] = vx;
         out[t * 4 + 1] = vy;
-        out[t * 4 + 2] = S[t * 3 + 2] * f.inv_N;
+        out[t * 4 + 2] = S[0][t * 3 + 2] * f.inv_N;
         out[t * 4 + 3] = -qe * f.n[t] * vx;
     }
 }
 
-// maximum over the cells of each node's histogram
-__global__ void k_hist_max(const uint32_t *H, int64_t cells, uint32_t *out)
+// Maximum over the cells of each node's histogram into out[q] (zeroed before): gridDim = (nodes,
+// blocks per node).  One block per node took 14-33 us for 240 x 240 cells, memory latency of its 225
+// rounds of loads; 3-5 us over kHistMaxBlocks blocks with four cells per load.
+constexpr int kHistMaxBlocks = 16;
+__global__ void __launch_bounds__(256) k_hist_max(const uint32_t *H, int64_t cells, uint32_t *out)
 {
-    __shared__ uint32_t sm[32];
     const uint32_t *h = H + (int64_t)blockIdx.x * cells;
+    const int64_t t0 = (int64_t)blockIdx.y * blockDim.x + threadIdx.x, nt = (int64_t)gridDim.y * blockDim.x;
     uint32_t m = 0;
-    for (int64_t j = threadIdx.x; j < cells; j += blockDim.x) m = max(m, h[j]);
-#pragma unroll
-    for (int o = 16; o > 0; o >>= 1) m = max(m, __shfl_xor_sync(0xffffffffu, m, o));
-    if ((threadIdx.x & 31) == 0) sm[threadIdx.x >> 5] = m;
-    __syncthreads();
-    if (threadIdx.x < 32) {
-        m = (threadIdx.x < (blockDim.x >> 5)) ? sm[threadIdx.x] : 0u;
-#pragma unroll
-        for (int o = 16; o > 0; o >>= 1) m = max(m, __shfl_xor_sync(0xffffffffu, m, o));
-        if (threadIdx.x == 0) out[blockIdx.x] = m;
+    if ((reinterpret_cast<uintptr_t>(h) & 15) == 0) {   // (uniform: a node's cells may start at any word)
+        for (int64_t j = t0; j < cells / 4; j += nt) {
+            const uint4 v = reinterpret_cast<const uint4 *>(h)[j];
+            m = max(max(m, max(v.x, v.y)), max(v.z, v.w));
+        }
+        for (int64_t j = (cells & ~(int64_t)3) + t0; j < cells; j += nt) m = max(m, h[j]);
+    } else {
+        for (int64_t j = t0; j < cells; j += nt) m = max(m, h[j]);
     }
+    m = __reduce_max_sync(0xffffffffu, m);
+    if ((threadIdx.x & 31) == 0 && m) atomicMax(&out[blockIdx.x], m);
+}
+
+static cudaError_t launch_hist_max(const uint32_t *H, int Q, int64_t cells, uint32_t *out, cudaStream_t s)
+{
+    cudaError_t e = cudaMemsetAsync(out, 0, (size_t)Q * 4, s);
+    if (e != cudaSuccess) return e;
+    k_hist_max<<<dim3((unsigned)Q, kHistMaxBlocks), 256, 0, s>>>(H, cells, out);
+    count_launch();
+    return cudaGetLastError();
 }
 
 // Fixed-order reduction of g1 block partials (no second set) into one moment record of ctx's
@@ -620,7 +638,7 @@ static pgc_status check_config(const pgc_config *c, Layout *L, std::string *msg)
     L->off_series = take((size_t)c->max_outputs * L->rec_len * 8);
     L->off_recon = take((size_t)c->Nk * c->Nk * 4);
     L->off_tmpmax = take(4);
-    L->off_obs = take((size_t)(kObsGrid * kObsZ * 3 + kObsZ * 4) * 8);
+    L->off_obs = take((size_t)(kObsGrid * kObsZ * 3 + kObsBatch * kObsZ * 4) * 8);
     L->off_colsum = take((size_t)64 * 3 * 8);
     L->off_fdtab = take(kFdTableBytes);
     L->off_edgetab = take(c->precision == PGC_FP64 ? (size_t)(c->n_theta_edge + 1) * kEdgeK * 8 : 0);
@@ -684,8 +702,8 @@ static pgc_status observe_current(pgc_ctx *ctx, bool record, bool set_nmax)
     if ((e = ctx->run->observe(cur, s)) != cudaSuccess) return cuda_fail(ctx, e, "observe");
     const int64_t cells = (int64_t)ctx->t.Nk * ctx->t.Nk;
     if (set_nmax) {
-        k_hist_max<<<ctx->t.Q, 256, 0, s>>>(ctx->b.hist + (int64_t)cur * ctx->b.hist_stride, cells, ctx->b.nmax);
-        count_launch();
+        if ((e = launch_hist_max(ctx->b.hist + (int64_t)cur * ctx->b.hist_stride, ctx->t.Q, cells, ctx->b.nmax, s)) != cudaSuccess)
+            return cuda_fail(ctx, e, "histogram maximum");
     }
     if (record) {
         if (ctx->T_out >= ctx->cfg.max_outputs) return fail(ctx, PGC_ENOMEM, "moment series full (max_outputs)");
@@ -698,7 +716,8 @@ static pgc_status observe_current(pgc_ctx *ctx, bool record, bool set_nmax)
         f.g1 = ctx->run->grid1();
         f.g2 = 0;
         f.g3 = 0;
-        k_finalize<<<1, kFinThreads, 0, s>>>(ctx->b.part1, nullptr, nullptr, f, ctx->series + ctx->T_out * ctx->rec_len);
+        k_finalize_cols<<<ctx->t.Q * 3, kFinColThreads, 0, s>>>(ctx->b.part1, nullptr, nullptr, f, ctx->colsum, ctx->b.qcount + 3,
+                                                                ctx->series + ctx->T_out * ctx->rec_len);
         count_launch();
         ctx->T_out++;
     }
@@ -837,8 +856,7 @@ pgc_status pgc_step(pgc_ctx *ctx, int64_t n_steps, int32_t moments_every)
     auto is_out = [&](int64_t n) { return moments_every > 0 && ((n + 1) % moments_every == 0); };
     auto hist_max = [&](int64_t n) {
         if (ctx->t.pauli_mode != PGC_PAULI_CURRENT_MAX) return;
-        k_hist_max<<<ctx->t.Q, 256, 0, s>>>(ctx->b.hist + (int64_t)(n % kHistBufs) * ctx->b.hist_stride, cells, ctx->b.nmax);
-        count_launch();
+        launch_hist_max(ctx->b.hist + (int64_t)(n % kHistBufs) * ctx->b.hist_stride, ctx->t.Q, cells, ctx->b.nmax, s);
     };
     // record of step n: phase-1 partials of step n (g1 blocks), phase-2 partials of step n (g2
     // blocks) and, when phase 2 of step n - 1 carried particles into step n, its partials of step
@@ -1117,9 +1135,7 @@ pgc_status pgc_reconstruct_f(pgc_ctx *ctx, const double *h_z, int32_t nz, uint32
         cudaError_t e = cudaMemsetAsync(ctx->b.recon_hist, 0, cells * 4, ctx->stream);
         if (e == cudaSuccess) e = ctx->run->hist_at(psi.data(), xs, ctx->b.recon_hist, ctx->stream);
         if (e == cudaSuccess) {
-            k_hist_max<<<1, 256, 0, ctx->stream>>>(ctx->b.recon_hist, cells, ctx->tmp_max);
-            count_launch();
-            e = cudaGetLastError();
+            e = launch_hist_max(ctx->b.recon_hist, 1, cells, ctx->tmp_max, ctx->stream);
         }
         if (e == cudaSuccess)
             e = cudaMemcpyAsync(h_hist + (size_t)j * cells, ctx->b.recon_hist, cells * 4, cudaMemcpyDeviceToHost, ctx->stream);
@@ -1140,6 +1156,7 @@ pgc_status pgc_observe_at(pgc_ctx *ctx, const double *h_z, int32_t nz, double *h
         if (!(h_z[j] >= -1.0 && h_z[j] <= 1.0)) return fail(ctx, PGC_EINVAL, "z outside [-1,1]");
     const HostTables &t = ctx->t;
     std::vector<double> psi((size_t)kObsZ * P), e0(kObsZ), xs(kObsZ);
+    int out0 = 0;   // first point whose result waits on the device (one copy per kObsBatch passes)
     for (int j0 = 0; j0 < nz; j0 += kObsZ) {
         const int nzc = std::min(kObsZ, nz - j0);
         ObsFin f{};
@@ -1160,12 +1177,15 @@ pgc_status pgc_observe_at(pgc_ctx *ctx, const double *h_z, int32_t nz, double *h
             f.inv_N = 1.0 / (double)ctx->b.N;
             f.nz = nzc;
             f.g = g;
-            k_obs_fin<<<1, 128, 0, ctx->stream>>>(ctx->obs_part, f, ctx->obs_out);
+            k_obs_fin<<<1, kObsZ * 3 * kObsFinSlots, 0, ctx->stream>>>(ctx->obs_part, f, ctx->obs_out + (size_t)(j0 - out0) * 4);
             count_launch();
             e = cudaGetLastError();
         }
-        if (e == cudaSuccess)
-            e = cudaMemcpyAsync(h_out + (size_t)j0 * 4, ctx->obs_out, (size_t)nzc * 4 * 8, cudaMemcpyDeviceToHost, ctx->stream);
+        const int done = j0 + nzc;
+        if (e == cudaSuccess && (done == nz || done - out0 == kObsBatch * kObsZ)) {
+            e = cudaMemcpyAsync(h_out + (size_t)out0 * 4, ctx->obs_out, (size_t)(done - out0) * 4 * 8, cudaMemcpyDeviceToHost, ctx->stream);
+            out0 = done;
+        }
         if (e != cudaSuccess) return cuda_fail(ctx, e, "observe_at");
     }
     cudaError_t e = cudaStreamSynchronize(ctx->stream);

@@ -18,10 +18,10 @@
 // particle and node, where the iteration (fd_inverse) takes a 30-step FP32 bisection and about eight
 // FP64 evaluations of G (each an exp, two log1p, a division and a 12-term series).  The FP64 pipe of
 // this part issues two lanes per clock and SM, and bounds both.  Measured: the sampling of 500 000
-// particles at 36 nodes 208 -> 2.0 ms, of 1e6 particles at 6 nodes 56.2 -> 0.44 ms, its
-// sensitivities at 5e5 x 6 nodes 32.2 -> 0.5 ms; the table itself takes 39 us (a warp per
-// block: latency of four to five Newton steps).  Error of eps against extended precision: rms
-// 2.9e-16 (iteration: 4.1e-16) for eps0 in [0.05, 0.15] eV at eps_F = 0.4 eV, 300 K.
+// particles at 36 nodes 208 -> 1.6 ms, of 1e6 particles at 6 nodes 56.2 -> 0.44 ms, its
+// sensitivities at 5e5 x 6 nodes 32.2 -> 0.5 ms; the table itself takes 26 us (a warp per
+// block: latency of two FP64 Newton steps).  Error of eps against extended precision: rms
+// 3.9e-16 (iteration: 4.1e-16) for eps0 in [0.05, 0.15] eV at eps_F = 0.4 eV, 300 K.
 #pragma once
 
 #include <algorithm>
@@ -69,12 +69,12 @@ __host__ __device__ inline double fd_G(double w, double m, double &E)
 }
 
 // w with G(w) = g, safeguarded Newton on log G from the degenerate (w^2 / 2 = G(0) - g) or the
-// Boltzmann limit.  It ends when a step is at the rounding level, or small and no longer shrinking
-// (near w = 0 the rounding of G moves w by more than an ulp, and the steps never get below it).
+// Boltzmann limit, first in FP32 to a relative 1e-6, then in FP64 until a step's square is below
+// rounding.
 __host__ __device__ inline double fd_solve(double g, const FdInv &f)
 {
     const double m = f.m;
-    double E, lo = 0.0, hi = f.wtop, last = f.wtop;
+    double E, lo = 0.0, hi = f.wtop;
     double w;
     if (m > 0.0 && g > f.gmu) w = sqrt(fmax(2.0 * (f.gzero - g), 0.0));
     else {
@@ -82,6 +82,18 @@ __host__ __device__ inline double fd_solve(double g, const FdInv &f)
         w = m - (L < 30.0 ? log(expm1(L)) : L);
     }
     if (!(w > lo && w < hi)) w = 0.5 * (lo + hi);
+    {   // the FP32 root: two iterations of the slow FP64 functions are left
+        const float gf = (float)g, mf = (float)m;
+        float x = (float)w;
+        for (int it = 0; it < 7; ++it) {
+            const float b = x - mf, ex = expf(-fabsf(b)), l = log1pf(ex), l2 = l * l;
+            const float li = l + 0.25f * l2 + l * l2 * (0.027777778f + l2 * (-2.7777778e-4f + l2 * 4.7241118e-6f));
+            const float G = b >= 0.0f ? x * l + li : x * l - b * (mf + 0.5f * b) + 1.6449341f - li;
+            const float E = b >= 0.0f ? 1.0f + 1.0f / ex : 1.0f + ex;
+            x = fmaxf(x + log1pf((G - gf) / gf) * G * E / x, 0.5f * x);
+        }
+        if (x > (float)lo && x < (float)hi) w = (double)x;   // (false for NaN)
+    }
     for (int it = 0; it < 80; ++it) {
         const double G = fd_G(w, m, E), d = (G - g) / g;
         if (d == 0.0) break;
@@ -90,8 +102,7 @@ __host__ __device__ inline double fd_solve(double g, const FdInv &f)
         if (!(wn >= lo && wn <= hi)) wn = 0.5 * (lo + hi);
         const double step = fabs(wn - w);
         w = wn;
-        if (step <= 3e-16 * w || (step <= 1e-7 * w && step >= 0.25 * last)) break;
-        last = step;
+        if (step <= 1e-8 * fmin(w, 1.0)) break;   // the next one would be its square (exp(w) sets the scale above 1)
     }
     return w;
 }

@@ -323,8 +323,8 @@ public:
         ReconArgs<P, Q, R> z;
         for (int h = 0; h < P; ++h) z.psi[h] = psi[h];
         z.lkx = (R)(t_.Lk - xs);
-        int blocks = (int)std::min<int64_t>((b_.N + 255) / 256, 4096);
-        k_hist_at<P, Q, R><<<blocks, 256, 0, s>>>(args_, z, out);
+        int blocks = (int)std::min<int64_t>((b_.N + 511) / 512, kHistAtGrid);
+        k_hist_at<P, Q, R><<<blocks, 512, 0, s>>>(args_, z, out);
         count_launch();
         return cudaGetLastError();
     }
