@@ -609,6 +609,16 @@ __device__ __forceinline__ void store_vec(R *p, const R v[PPT])
     }
 }
 
+// The rolled node loop of the large one-dimensional FP32 shapes reads its weights from a shared-memory copy
+// (rows padded to 16 bytes, two weights per load, four nodes' sums in flight): indexed reads of the
+// parameter bank, one weight each, and one dependent sum at a time bounded it (21 nodes, 1e4
+// particles: 17.3 us a launch; 15.8 us).
+template <int P, int Q, typename R> struct StagePsi {
+    static constexpr bool value = P * Q > 64 && !TensorShape<P, Q>::value && sizeof(R) == 4;
+    static constexpr int row = (P + 1) & ~1;
+    static constexpr int elems = value ? Q * row : 2;
+};
+
 // Everything phase 1 needs about one ensemble (one case of a batch).
 template <typename R>
 struct P1Target {
@@ -664,7 +674,7 @@ template <int P, int Q, typename R, int W = HistWin<P, Q, R>::W, int PPT = Phase
 __device__ __forceinline__ void phase1_pass(const Phys<R> &ph, const Nodes<P, Q, R> &nd, const P1Target<R> &t,
                                             int64_t i0, uint32_t *swin, int win_r0, bool use_win, float kk_in, bool out_step,
                                             typename MomAcc<R>::T *smom_warp, uint32_t *aside, int &n_aside,
-                                            unsigned int &oog)
+                                            unsigned int &oog, const unsigned long long *spsi = nullptr)
 {
     const int lane = threadIdx.x & 31;
     const int64_t NN = (int64_t)ph.Nk * ph.Nk;
@@ -717,10 +727,26 @@ __device__ __forceinline__ void phase1_pass(const Phys<R> &ph, const Nodes<P, Q,
             if constexpr (sizeof(R) == 4) {
                 const F2 magic2 = window_magic(win_r0);
                 KkMax km;
-                recon_all(nd, cx[e], cy[e], [&](int q, R kx, R ky) {
-                    cell[q] = window_code<W>(kx, ky, nd.lk2[q], inv2, magic2);
-                    km.add(q, Q, knorm2(kx, ky));
-                });
+                if constexpr (StagePsi<P, Q, R>::value) {
+#pragma unroll 4
+                    for (int q = 0; q < Q; ++q) {
+                        const ulonglong2 *w = reinterpret_cast<const ulonglong2 *>(spsi + q * StagePsi<P, Q, R>::row);
+                        F2 s2 = f2_pack(0.f, 0.f);
+#pragma unroll
+                        for (int h = 0; h < P; ++h) s2 = f2_fma(f2_pack(cx[e][h], cy[e][h]), (h & 1) ? w[h >> 1].y : w[h >> 1].x, s2);
+                        float kx, ky;
+                        f2_unpack(s2, kx, ky);
+                        cell[q] = window_code<W>(kx, ky, nd.lk2[q], inv2, magic2);
+                        const float kk = knorm2(kx, ky);
+                        km.m = fmaxf(km.m, kk);
+                        km.n = max3_nan(km.n, kk, kk);
+                    }
+                } else {
+                    recon_all(nd, cx[e], cy[e], [&](int q, R kx, R ky) {
+                        cell[q] = window_code<W>(kx, ky, nd.lk2[q], inv2, magic2);
+                        km.add(q, Q, knorm2(kx, ky));
+                    });
+                }
                 in_window = km.n <= kk_in;   // (false for NaN)
                 maybe = screen_maybe(ph, nd, km.m, r.x);
             } else {
@@ -897,6 +923,13 @@ __device__ __forceinline__ void phase1_block(const StepArgs<P, Q, R> &a, int bid
     const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
     uint32_t *aside = s_aside[warp];
     int n_aside = 0;
+    using SP = StagePsi<P, Q, R>;
+    __shared__ __align__(16) unsigned long long spsi[SP::elems];
+    if constexpr (SP::value)
+        for (int j = threadIdx.x; j < Q * P; j += blockDim.x) {
+            const float w = a.nd_dev ? a.nd_dev->psi[j] : a.nd.psi[j];
+            spsi[(j / P) * SP::row + j % P] = f2_pack(w, w).v;
+        }
     if (a.use_win) clear_window<Q, HistWin<P, Q, R>::W>(swin);
     if (a.out_step)
         for (int j = lane; j < Q * 3; j += 32) acc_zero(smom[warp][j]);
@@ -952,13 +985,13 @@ __device__ __forceinline__ void phase1_block(const StepArgs<P, Q, R> &a, int bid
             if (tl >= ntiles) break;
             guard_window();
             phase1_pass<P, Q, R>(a.ph, a.nd, t, tl * tile + (int64_t)threadIdx.x * PPT, swin, a.win_r0,
-                                 a.use_win != 0, a.kk_in, a.out_step != 0, smom[warp], aside, n_aside, oog);
+                                 a.use_win != 0, a.kk_in, a.out_step != 0, smom[warp], aside, n_aside, oog, spsi);
         }
     } else {
         for (int64_t base = (int64_t)bid * tile; base < a.N; base += (int64_t)nb * tile) {
             guard_window();
             phase1_pass<P, Q, R>(a.ph, a.nd, t, base + (int64_t)threadIdx.x * PPT, swin, a.win_r0, a.use_win != 0, a.kk_in,
-                                 a.out_step != 0, smom[warp], aside, n_aside, oog);
+                                 a.out_step != 0, smom[warp], aside, n_aside, oog, spsi);
         }
     }
     if (n_aside > 0)
