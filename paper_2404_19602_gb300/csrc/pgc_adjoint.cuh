@@ -5,12 +5,12 @@
 // outcomes, the trapezoid segment of the edge angle and all histogram cells; the random numbers
 // are the forward run's (Philox counters are recomputed, nothing is stored).  The forward run
 // keeps a checkpoint (state + histogram f^n) every K steps; the backward pass replays each
-// segment with the forward kernels, keeping the K states and histograms of the segment, then
-// walks the segment backwards:
-//   k_adj_screen  (every particle): adds the moment term of time n+1 to lambda, redoes the
-//                 phase-1 flight-time screen of step n (same code, same decision), and for the
-//                 particles that cannot have collided adds the drift term -d(dhat)/d(theta).lambda;
-//                 the others are queued;
+// segment with the forward kernels, keeping of each step f^n, the collider queue and the colliders'
+// states (the whole state where a moment term needs it), then walks the segment backwards:
+//   k_adj_screen  (every particle): adds the moment term of time n+1 to lambda (on moment steps), and for
+//                 the particles that cannot have collided in step n (not marked by the replay) adds the
+//                 drift term -d(dhat)/d(theta).lambda.  Without a moment term it reads the bitmap and
+//                 the planes of lambda that the drift term needs, nothing else;
 //   k_adj_collide (queued, lanes <-> nodes as in the forward collider kernel): replays the event
 //                 chain of step n bit for bit, then applies the transposed Jacobians of the
 //                 projection, the final-state maps h^l and the reconstruction, event by event from
@@ -28,23 +28,28 @@
 namespace pgc {
 
 constexpr int NTH = 4;  // E_lo, E_hi, eps0_lo, eps0_hi
+constexpr int kAdjKeep = 4;  // events of a particle kept between the forward replay and the backward walk
 
 template <int P, int Q, typename R>
 struct AdjArgs {
     Phys<R> ph;
     Nodes<P, Q, R> nd;
-    const R *khat_n;          // state before step n (pre-drift), [2][P][ld]
+    const R *khat_n;          // compact: drifted states of the queue's particles, column j for entry j;
+                              // else the state before step n (pre-drift); [2][P][ld]
     const R *khat_n1;         // state after step n (moment term of time n+1)
+    int32_t compact;
+    const uint32_t *mark;     // bitmap of the particles queued at step n
     R *lam;                   // adjoint of the state, [2][P][ld]
     const uint32_t *Hn;       // f^n
     const uint32_t *nmax;
-    uint32_t *queue, *qcount;
+    const uint32_t *queue, *qcount;
     double *grad;             // [NTH], accumulated
     int64_t N, ld;
     uint32_t key0, key1, stream_id, step;
     int32_t inject;           // time n+1 is an output in the window
     double dLdJ[Q];           // dL/dJ_q at time n+1 (objective weights / number of outputs included)
     double ddhat[NTH][P];     // d dhat_h / d theta_t (per step)
+    uint32_t ddmask;          // coefficients h with a non-zero ddhat
     double de0[Q][NTH];       // d eps0_q / d theta_t
     double nq[Q], dnq[Q];     // density and d n / d eps0 at the nodes (m^-2)
     double cJ;                // -e vF / N : J_q = cJ n_q sum_i vhat
@@ -92,16 +97,43 @@ k_adj_screen(const __grid_constant__ AdjArgs<P, Q, R> a)
 #pragma unroll
     for (int q = 0; q < SQ; ++q) { svh[q] = (R)0; sdve[q] = (R)0; }
     const int64_t stride = (int64_t)gridDim.x * blockDim.x;
-    const int lane = threadIdx.x & 31;
-    for (int64_t base = (int64_t)blockIdx.x * blockDim.x; base < a.N; base += stride) {
-        const int64_t i = base + threadIdx.x;
-        bool maybe = false;
-        if (i < a.N) {
-            R lx[P], ly[P];
+    if constexpr (kSums) {
+        if (!a.inject) {
+            // no moment term: the drift term's planes of lambda over the unmarked particles, four loads in
+            // flight (one by one the loop is a chain of memory latencies, 14 us at 5e5 particles)
 #pragma unroll
             for (int h = 0; h < P; ++h) {
-                lx[h] = a.lam[(int64_t)h * a.ld + i];
-                ly[h] = a.lam[(int64_t)(P + h) * a.ld + i];
+                if (!(a.ddmask & (1u << h))) continue;
+                const R *l = a.lam + (int64_t)h * a.ld;
+                for (int64_t i = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; i < a.N; i += 4 * stride) {
+                    R v[4];
+                    bool ok[4];
+#pragma unroll
+                    for (int u = 0; u < 4; ++u) {
+                        const int64_t j = i + u * stride;
+                        ok[u] = j < a.N && !((a.mark[j >> 5] >> (j & 31)) & 1u);
+                        v[u] = j < a.N ? l[j] : (R)0;
+                    }
+#pragma unroll
+                    for (int u = 0; u < 4; ++u)
+                        if (ok[u]) slx[h] += v[u];
+                }
+            }
+        }
+    }
+    for (int64_t base = (int64_t)blockIdx.x * blockDim.x; base < a.N && (!kSums || a.inject); base += stride) {
+        const int64_t i = base + threadIdx.x;
+        if (i < a.N) {
+            R lx[P], ly[P];
+            if (a.inject) {
+#pragma unroll
+                for (int h = 0; h < P; ++h) {
+                    lx[h] = a.lam[(int64_t)h * a.ld + i];
+                    ly[h] = a.lam[(int64_t)(P + h) * a.ld + i];
+                }
+            } else {
+#pragma unroll
+                for (int h = 0; h < P; ++h) lx[h] = (a.ddmask & (1u << h)) ? a.lam[(int64_t)h * a.ld + i] : (R)0;
             }
             if (a.inject) {
                 // dL/dk(z_q) = dL/dJ_q cJ n_q d vhat/dk,  vhat = hvF kx / eps(k, eps0_q)  (in R)
@@ -144,22 +176,7 @@ k_adj_screen(const __grid_constant__ AdjArgs<P, Q, R> a)
                     a.lam[(int64_t)(P + h) * a.ld + i] = ly[h];
                 }
             }
-            // the flight-time screen of phase 1 at step n (identical arithmetic)
-            R cx[P], cy[P];
-#pragma unroll
-            for (int h = 0; h < P; ++h) {
-                cx[h] = a.khat_n[(int64_t)h * a.ld + i];
-                cy[h] = a.khat_n[(int64_t)(P + h) * a.ld + i];
-                if (nd.drift_mask & (1u << h)) cx[h] -= nd.dhat[h];
-            }
-            R kkmax = (R)0;
-            recon_all(nd, cx, cy, [&](int, R kx, R ky) { kkmax = fmax(kkmax, kx * kx + ky * ky); });
-            const U4 r = philox4x32_10((uint32_t)i, a.stream_id, a.step, 0u, a.key0, a.key1);
-            const R lnxi = -rlog<R>(u01<R>(r.x));
-            const R emax = rsqrt_<R>(ph.hvF2 * kkmax + nd.eps0_max * nd.eps0_max);
-            const R gub = ph.alpha1 * rate_bound(ph, emax, nd.eps0_max) * (R)1.0001;
-            maybe = lnxi < gub * ph.dt;
-            if (!maybe) {  // lambda* = lambda: drift term -sum_h d dhat_h/d theta lambda_x,h
+            if (!((a.mark[i >> 5] >> (i & 31)) & 1u)) {  // lambda* = lambda: drift term -sum_h d dhat_h/d theta lambda_x,h
                 if constexpr (kSums) {
 #pragma unroll
                     for (int h = 0; h < P; ++h) slx[h] += lx[h];
@@ -168,19 +185,12 @@ k_adj_screen(const __grid_constant__ AdjArgs<P, Q, R> a)
                     for (int t = 0; t < NTH; ++t) {
                         double s = 0.0;
 #pragma unroll
-                        for (int h = 0; h < P; ++h) s += a.ddhat[t][h] * (double)lx[h];
+                        for (int h = 0; h < P; ++h)
+                            if (a.ddmask & (1u << h)) s += a.ddhat[t][h] * (double)lx[h];
                         g[t] -= s;
                     }
                 }
             }
-        }
-        const unsigned int mask = __ballot_sync(0xffffffffu, maybe);
-        if (mask) {
-            const int leader = __ffs(mask) - 1;
-            uint32_t basepos = 0;
-            if (lane == leader) basepos = atomicAdd(a.qcount, (uint32_t)__popc(mask));
-            basepos = __shfl_sync(0xffffffffu, basepos, leader);
-            if (maybe) a.queue[basepos + __popc(mask & ((1u << lane) - 1u))] = (uint32_t)i;
         }
     }
     if constexpr (kSums) {
@@ -188,7 +198,8 @@ k_adj_screen(const __grid_constant__ AdjArgs<P, Q, R> a)
         for (int t = 0; t < NTH; ++t) {
             double s = 0.0;
 #pragma unroll
-            for (int h = 0; h < P; ++h) s += a.ddhat[t][h] * (double)slx[h];
+            for (int h = 0; h < P; ++h)
+                if (a.ddmask & (1u << h)) s += a.ddhat[t][h] * (double)slx[h];
             g[t] -= s;
         }
         if (a.inject)
@@ -293,20 +304,22 @@ __device__ void fs_jacobian(const Phys<R> &ph, int l, R kx, R ky, EventAngles<R>
 // layout; an event that changes no node leaves the coefficients, rates and majorant untouched)
 // for at most `stop` events; on return cx/cy/kx/ky hold the state before event `stop` (or the
 // final state), and *nev the number of events the loop would run.  The mechanism of every node
-// at event `stop` is returned in l_out[] (6 = unchanged).
-template <int P, int Q, typename R>
+// at event `stop` is returned in l_out[] (6 = unchanged).  rec(e, s, kx, ky, l, r) is called for every
+// event e applied and node slot s with the node value before it and its mechanism (6 = unchanged).
+template <int P, int Q, typename R, typename F>
 __device__ __forceinline__ void replay_events(const Phys<R> &ph, const Nodes<P, Q, R> &nd, const AdjArgs<P, Q, R> &a,
-                                              int64_t i, int r, unsigned gmask, int stop, R cx[P], R cy[P],
+                                              int64_t i, int64_t j, int r, unsigned gmask, int stop, R cx[P], R cy[P],
                                               R kx[GroupOf<Q>::NPL], R ky[GroupOf<Q>::NPL], int *nev,
-                                              int l_out[GroupOf<Q>::NPL], U4 *r_out, R *red)
+                                              int l_out[GroupOf<Q>::NPL], U4 *r_out, R *red, F &&rec)
 {
     constexpr int G = GroupOf<Q>::G, NPL = GroupOf<Q>::NPL;
     const int64_t NN = (int64_t)ph.Nk * ph.Nk;
+    const int64_t col = a.compact ? j : i;
 #pragma unroll
     for (int h = 0; h < P; ++h) {
-        cx[h] = a.khat_n[(int64_t)h * a.ld + i];
-        cy[h] = a.khat_n[(int64_t)(P + h) * a.ld + i];
-        if (nd.drift_mask & (1u << h)) cx[h] -= nd.dhat[h];
+        cx[h] = a.khat_n[(int64_t)h * a.ld + col];
+        cy[h] = a.khat_n[(int64_t)(P + h) * a.ld + col];
+        if (!a.compact && (nd.drift_mask & (1u << h))) cx[h] -= nd.dhat[h];
     }
 #pragma unroll
     for (int s = 0; s < NPL; ++s) {
@@ -344,7 +357,7 @@ __device__ __forceinline__ void replay_events(const Phys<R> &ph, const Nodes<P, 
                 l_out[s] = 6;
                 if (q >= Q) continue;
                 R g[6];
-                rates6(ph, kx[s], ky[s], nd.eps0[q], g);
+                rates6<false>(ph, kx[s], ky[s], nd.eps0[q], g);
                 int l = 6;
                 R cum = (R)0;
 #pragma unroll
@@ -374,7 +387,9 @@ __device__ __forceinline__ void replay_events(const Phys<R> &ph, const Nodes<P, 
             const int q = r + s * G;
             if (q >= Q) continue;
             R g[6];
-            rates6(ph, kx[s], ky[s], nd.eps0[q], g);
+            // (rounded as this replay's selection always was: a mechanism boundary hit to the last bit goes
+            // one way in ~1e-8 of the events, and one event moves a gradient of 5e5 particles by 1e-6)
+            rates6<false>(ph, kx[s], ky[s], nd.eps0[q], g);
             int l = 6;
             R cum = (R)0;
 #pragma unroll
@@ -382,7 +397,7 @@ __device__ __forceinline__ void replay_events(const Phys<R> &ph, const Nodes<P, 
                 cum += g[m];
                 if (l == 6 && target < cum) l = m;
             }
-            if (l == 6) continue;
+            if (l == 6) { rec(e, s, kx[s], ky[s], 6, rr); continue; }
             R nkx, nky;
             final_state<8>(ph, l, kx[s], ky[s], nd.eps0[q], ang, &nkx, &nky);
             bool accept = true;
@@ -390,6 +405,7 @@ __device__ __forceinline__ void replay_events(const Phys<R> &ph, const Nodes<P, 
                 const int cl = cell_of(ph, nd.lkx[q], nkx + nd.dq[q], nky);
                 if (cl >= 0) accept = pauli_accept(a.Hn[(int64_t)q * NN + cl], a.nmax[q], rr.z);
             }
+            rec(e, s, kx[s], ky[s], accept ? l : 6, rr);
             if (accept) { kx[s] = nkx; ky[s] = nky; changed = true; }
         }
         if (group_any<G>(changed, gmask)) {   // the forward's projection, reconstruction and majorant
@@ -423,6 +439,13 @@ k_adj_collide(const __grid_constant__ AdjArgs<P, Q, R> a)
     __syncthreads();
     const Phys<R> &ph = *reinterpret_cast<const Phys<R> *>(sph);
     const Nodes<P, Q, R> &nd = *reinterpret_cast<const Nodes<P, Q, R> *>(snd);
+    // The first kAdjKeep events of a lane's particle as its forward replay passes them: a particle has
+    // one or two, and replaying from the start to each event of the backward walk doubled the kernel (6 nodes,
+    // 5e5 particles: 37.6 us a launch; 26.1 us kept).  Later events are replayed.
+    __shared__ typename Pair<R>::T s_k[kAdjKeep][NPL][kPhase2Threads];
+    __shared__ unsigned char s_l[kAdjKeep][NPL][kPhase2Threads];
+    __shared__ uint32_t s_w[kAdjKeep][kPhase2Threads];
+    const int tid = threadIdx.x;
     const uint32_t count = *a.qcount;
     const int lane = threadIdx.x & 31;
     const int r = lane % G;
@@ -439,11 +462,32 @@ k_adj_collide(const __grid_constant__ AdjArgs<P, Q, R> a)
         }
         R cx[P], cy[P], kx[NPL], ky[NPL];
         int nev = 0, lsel[NPL];
-        U4 rr;
-        replay_events(ph, nd, a, i, r, gmask, 1 << 30, cx, cy, kx, ky, &nev, lsel, &rr, sred);
+        U4 rr{0u, 0u, 0u, 0u};
+        replay_events(ph, nd, a, i, j, r, gmask, 1 << 30, cx, cy, kx, ky, &nev, lsel, &rr, sred,
+                      [&](int e, int s, R x, R y, int l, const U4 &w) {
+                          if (e >= kAdjKeep) return;
+                          s_k[e][s][tid].x = x;
+                          s_k[e][s][tid].y = y;
+                          s_l[e][s][tid] = (unsigned char)l;
+                          s_w[e][tid] = w.w;
+                      });
         for (int e = nev - 1; e >= 0; --e) {
-            int dummy;
-            replay_events(ph, nd, a, i, r, gmask, e, cx, cy, kx, ky, &dummy, lsel, &rr, sred);
+            if (e < kAdjKeep) {   // (each lane reads what it wrote; lanes without a node wrote nothing)
+#pragma unroll
+                for (int s = 0; s < NPL; ++s) {
+                    lsel[s] = 6;
+                    if (r + s * G < Q) {
+                        kx[s] = s_k[e][s][tid].x;
+                        ky[s] = s_k[e][s][tid].y;
+                        lsel[s] = s_l[e][s][tid];
+                        rr.w = s_w[e][tid];
+                    }
+                }
+            } else {
+                int dummy;
+                replay_events(ph, nd, a, i, j, r, gmask, e, cx, cy, kx, ky, &dummy, lsel, &rr, sred,
+                              [](int, int, R, R, int, const U4 &) {});
+            }
             bool any = false;
 #pragma unroll
             for (int s = 0; s < NPL; ++s) any |= lsel[s] < 6;
@@ -493,7 +537,8 @@ k_adj_collide(const __grid_constant__ AdjArgs<P, Q, R> a)
             for (int t = 0; t < NTH; ++t) {
                 double s = 0.0;
 #pragma unroll
-                for (int h = 0; h < P; ++h) s += a.ddhat[t][h] * (double)lx[h];
+                for (int h = 0; h < P; ++h)
+                    if (a.ddmask & (1u << h)) s += a.ddhat[t][h] * (double)lx[h];
                 g[t] -= s;
             }
         }
@@ -574,15 +619,16 @@ k_adj_init(const __grid_constant__ AdjArgs<P, Q, R> a, const __grid_constant__ A
 // ------------------------------------------------------------------------------------------
 struct AdjBuffers {
     void *lam = nullptr;
-    uint32_t *queue = nullptr, *qcount = nullptr;
     double *grad = nullptr;
 };
 
 class AdjRunner {
 public:
     virtual ~AdjRunner() {}
-    // backward step n: moment term of time n+1 (if inject), then the map of step n
-    virtual cudaError_t backward_step(const void *khat_n, const void *khat_n1, const uint32_t *Hn, int64_t n,
+    // backward step n: moment term of time n+1 (if inject, from the state khat_n1), then the map of
+    // step n over its queue, the colliders' states compact or in the whole state khat_n
+    virtual cudaError_t backward_step(const void *khat_n, bool compact, const void *khat_n1, const uint32_t *Hn,
+                                      const uint32_t *mark, const uint32_t *queue, const uint32_t *count, int64_t n,
                                       bool inject, const double *dLdJ, cudaStream_t s) = 0;
     virtual cudaError_t init_term(cudaStream_t s) = 0;
 };
@@ -597,8 +643,6 @@ public:
         a_.nd = proto.args().nd;
         a_.lam = static_cast<R *>(ab.lam);
         a_.nmax = b.nmax;
-        a_.queue = ab.queue;
-        a_.qcount = ab.qcount;
         a_.grad = ab.grad;
         a_.N = b.N;
         a_.ld = b.ld;
@@ -620,11 +664,19 @@ public:
             const double rho = e0 / (1.0 + std::exp(std::fmin((e0 - t.mu) / t.kT, 700.0)));
             a_.dnq[q] = -2.0 / (kPi * t.hvF * t.hvF) * rho * 1.0e18;
         }
+        double ddmax = 0.0;
         for (int k = 0; k < NTH; ++k)
             for (int h = 0; h < P; ++h) {
                 double sacc = 0.0;
                 for (int q = 0; q < Q; ++q) sacc += t.wpsi[(size_t)q * P + h] * dEq_[q][k] * 1.0e-7 * t.dt / t.hbar_fs;
                 a_.ddhat[k][h] = sacc;
+                ddmax = std::max(ddmax, std::fabs(sacc));
+            }
+        // as for the drift itself: the field is affine in z, other entries are quadrature round-off
+        for (int k = 0; k < NTH; ++k)
+            for (int h = 0; h < P; ++h) {
+                if (std::fabs(a_.ddhat[k][h]) <= 1e-13 * ddmax) a_.ddhat[k][h] = 0.0;
+                if (a_.ddhat[k][h] != 0.0) a_.ddmask |= 1u << h;
             }
         for (int i = 0; i < Q * P; ++i) ia_.wpsi[i] = t.wpsi[i];
         for (int q = 0; q < Q; ++q) {
@@ -643,23 +695,26 @@ public:
                 ia_.ie0[q] = 1.0 / (1.0 + std::exp(w0 - ia_.fd.m));
             }
         }
-        int per_sm = 0;
-        cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, k_adj_screen<P, Q, R>, 256, 0);
+        // the grid groups the FP32 partial sums of the gradient's drift term: fixed, not by occupancy
+        const int per_sm = P == 1 ? (sizeof(R) == 4 ? 8 : 4) : (P <= 8 ? 2 : 1);
         grid_ = (int)std::max<int64_t>(1, std::min<int64_t>((b.N + 255) / 256, (int64_t)num_sms * std::max(per_sm, 1)));
     }
 
-    cudaError_t backward_step(const void *khat_n, const void *khat_n1, const uint32_t *Hn, int64_t n, bool inject,
+    cudaError_t backward_step(const void *khat_n, bool compact, const void *khat_n1, const uint32_t *Hn,
+                              const uint32_t *mark, const uint32_t *queue, const uint32_t *count, int64_t n, bool inject,
                               const double *dLdJ, cudaStream_t s) override
     {
         AdjArgs<P, Q, R> a = a_;
         a.khat_n = static_cast<const R *>(khat_n);
+        a.compact = compact ? 1 : 0;
         a.khat_n1 = static_cast<const R *>(khat_n1);
         a.Hn = Hn;
+        a.mark = mark;
+        a.queue = queue;
+        a.qcount = count;
         a.step = (uint32_t)n;
         a.inject = inject ? 1 : 0;
         for (int q = 0; q < Q; ++q) a.dLdJ[q] = inject ? dLdJ[q] : 0.0;
-        cudaError_t e = cudaMemsetAsync(ab_.qcount, 0, sizeof(uint32_t), s);
-        if (e != cudaSuccess) return e;
         k_adj_screen<P, Q, R><<<grid_, 256, 0, s>>>(a);
         k_adj_collide<P, Q, R><<<kGrid2, kPhase2Threads, 0, s>>>(a);
         count_launch(2);

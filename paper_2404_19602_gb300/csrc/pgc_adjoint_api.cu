@@ -35,8 +35,8 @@ namespace {
 struct AdjLayout {
     int64_t nseg = 0;
     size_t state = 0, hist1 = 0;
-    size_t ckpt_state = 0, ckpt_hist = 0, replay_state = 0, replay_hist = 0, stack_state = 0, stack_hist = 0, lam = 0,
-           queue = 0, qcount = 0, counters = 0, part1 = 0, part2 = 0, aqueue = 0, aqcount = 0, grad = 0, total = 0;
+    size_t ckpt_state = 0, ckpt_hist = 0, replay_state = 0, stack_state = 0, stack_hist = 0, lam = 0,
+           queue = 0, qcount = 0, counters = 0, part1 = 0, part2 = 0, marks = 0, kept_queue = 0, kept_count = 0, grad = 0, total = 0;
 };
 
 int64_t rup(int64_t x, int64_t m) { return (x + m - 1) / m * m; }
@@ -55,17 +55,17 @@ pgc_status adj_layout(const pgc_ctx *ctx, int64_t n_steps, int32_t K, AdjLayout 
     L->ckpt_state = take((size_t)L->nseg * L->state);
     L->ckpt_hist = take((size_t)L->nseg * L->hist1);
     L->replay_state = take(L->state);
-    L->replay_hist = take((size_t)kHistBufs * ctx->b.hist_stride * 4);
-    L->stack_state = take((size_t)(K + 1) * L->state);
-    L->stack_hist = take((size_t)K * L->hist1);
+    L->stack_state = take((size_t)(K + 1) * L->state);   // slot n: the state at time n, or step n's colliders
+    L->stack_hist = take((size_t)(K + 1) * L->hist1);
     L->lam = take(L->state);
     L->queue = take((size_t)ctx->b.N * 4);
     L->qcount = take(8 * 4);
     L->counters = take(8 * 8);
     L->part1 = take((size_t)kMaxGrid1 * Q * 3 * 8);
     L->part2 = take((size_t)kGrid2Max * Q * 3 * 8);   // the replay runs the forward phase-2 grid
-    L->aqueue = take((size_t)ctx->b.N * 4);
-    L->aqcount = take(4 * 4);
+    L->marks = take((size_t)K * ctx->b.mark_words * 4);
+    L->kept_queue = take((size_t)K * ctx->b.N * 4);
+    L->kept_count = take((size_t)K * 4);
     L->grad = take(NTH * 8);
     L->total = off;
     return PGC_OK;
@@ -204,7 +204,7 @@ pgc_status pgc_adjoint(pgc_ctx *ctx, int64_t n_steps, int32_t ckpt_every, int32_
     // ---- reverse sweep ----
     DevBuffers rb = ctx->b;  // the replay runs the forward kernels on the work buffers
     rb.state = w + L.replay_state;
-    rb.hist = (uint32_t *)(w + L.replay_hist);
+    rb.hist = (uint32_t *)(w + L.stack_hist);   // (step_replay passes each step's two histograms)
     rb.queue = (uint32_t *)(w + L.queue);
     rb.queue_stride = 0;   // one queue: the replay runs the two-launch form of the step
     rb.qcount = (uint32_t *)(w + L.qcount);
@@ -220,8 +220,6 @@ pgc_status pgc_adjoint(pgc_ctx *ctx, int64_t n_steps, int32_t ckpt_every, int32_
     Runner *replay = make_runner(ctx->t.P, Q, ctx->cfg.precision, ctx->t, rb, sms);
     AdjBuffers ab;
     ab.lam = w + L.lam;
-    ab.queue = (uint32_t *)(w + L.aqueue);
-    ab.qcount = (uint32_t *)(w + L.aqcount);
     ab.grad = (double *)(w + L.grad);
     AdjRunner *adj = make_adj_runner(ctx->t.P, Q, ctx->cfg.precision, ctx->t, ctx->b, ab, sms);
     if (!replay || !adj) { delete replay; delete adj; return afail(ctx, PGC_EUNSUPPORTED, "no adjoint kernel for this shape"); }
@@ -229,25 +227,27 @@ pgc_status pgc_adjoint(pgc_ctx *ctx, int64_t n_steps, int32_t ckpt_every, int32_
     if (e == cudaSuccess) e = cudaMemsetAsync(ab.grad, 0, NTH * 8, s);
     for (int64_t sgi = L.nseg - 1; sgi >= 0 && e == cudaSuccess; --sgi) {
         const int64_t n0 = sgi * K, n1 = std::min<int64_t>(n_steps, n0 + K);
+        // slot n of the stacks: f^n, and of the state what the backward step needs: the whole state at a
+        // time with a moment term, else the states of step n's colliders
+        auto slot = [&](int64_t n) { return w + L.stack_state + (n - n0) * L.state; };
+        auto hist = [&](int64_t n) { return (uint32_t *)(w + L.stack_hist + (n - n0) * L.hist1); };
+        auto whole = [&](int64_t n) { return !dLdJ[n].empty(); };
         e = cudaMemcpyAsync(rb.state, w + L.ckpt_state + sgi * L.state, stbytes, cudaMemcpyDeviceToDevice, s);
-        if (e == cudaSuccess) e = cudaMemsetAsync(rb.hist, 0, (size_t)kHistBufs * rb.hist_stride * 4, s);
-        if (e == cudaSuccess)
-            e = cudaMemcpyAsync(rb.hist + (int64_t)(n0 % kHistBufs) * rb.hist_stride, w + L.ckpt_hist + sgi * L.hist1, hbytes,
-                                cudaMemcpyDeviceToDevice, s);
+        if (e == cudaSuccess) e = cudaMemsetAsync(w + L.stack_hist, 0, (size_t)(n1 - n0 + 1) * L.hist1, s);
+        if (e == cudaSuccess) e = cudaMemsetAsync(w + L.marks, 0, (size_t)(n1 - n0) * ctx->b.mark_words * 4, s);
+        if (e == cudaSuccess) e = cudaMemcpyAsync(hist(n0), w + L.ckpt_hist + sgi * L.hist1, hbytes, cudaMemcpyDeviceToDevice, s);
         if (e == cudaSuccess) e = cudaMemsetAsync(rb.qcount, 0, 8 * 4, s);
+        auto mark = [&](int64_t n) { return (uint32_t *)(w + L.marks) + (n - n0) * ctx->b.mark_words; };
+        auto kq = [&](int64_t n) { return (uint32_t *)(w + L.kept_queue) + (n - n0) * ctx->b.N; };
+        auto kc = [&](int64_t n) { return (uint32_t *)(w + L.kept_count) + (n - n0); };
         for (int64_t n = n0; n < n1 && e == cudaSuccess; ++n) {
-            e = cudaMemcpyAsync(w + L.stack_state + (n - n0) * L.state, rb.state, stbytes, cudaMemcpyDeviceToDevice, s);
-            if (e == cudaSuccess)
-                e = cudaMemcpyAsync(w + L.stack_hist + (n - n0) * L.hist1, rb.hist + (int64_t)(n % kHistBufs) * rb.hist_stride, hbytes,
-                                    cudaMemcpyDeviceToDevice, s);
-            if (e == cudaSuccess) e = replay->step(n, false, s);
+            if (whole(n)) e = cudaMemcpyAsync(slot(n), rb.state, stbytes, cudaMemcpyDeviceToDevice, s);
+            if (e == cudaSuccess) e = replay->step_replay(n, hist(n), hist(n + 1), mark(n), whole(n) ? nullptr : slot(n), kq(n), kc(n), s);
         }
-        if (e == cudaSuccess)
-            e = cudaMemcpyAsync(w + L.stack_state + (n1 - n0) * L.state, rb.state, stbytes, cudaMemcpyDeviceToDevice, s);
+        if (e == cudaSuccess && whole(n1)) e = cudaMemcpyAsync(slot(n1), rb.state, stbytes, cudaMemcpyDeviceToDevice, s);
         for (int64_t n = n1 - 1; n >= n0 && e == cudaSuccess; --n) {
-            const bool inj = !dLdJ[n + 1].empty();
-            e = adj->backward_step(w + L.stack_state + (n - n0) * L.state, w + L.stack_state + (n + 1 - n0) * L.state,
-                                   (const uint32_t *)(w + L.stack_hist + (n - n0) * L.hist1), n, inj,
+            const bool inj = whole(n + 1);
+            e = adj->backward_step(slot(n), !whole(n), slot(n + 1), hist(n), mark(n), kq(n), kc(n), n, inj,
                                    inj ? dLdJ[n + 1].data() : nullptr, s);
         }
     }

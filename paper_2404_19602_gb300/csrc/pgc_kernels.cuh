@@ -1429,6 +1429,24 @@ __device__ __forceinline__ void stage(uint32_t *dst, const T &src)
     for (int j = threadIdx.x; j < (int)(sizeof(T) / 4); j += blockDim.x) dst[j] = s[j];
 }
 
+// The queue of a step and, if save is non-NULL, the queued particles' coefficients before their collisions
+// (column j of [2P][ld] for queue entry j), for the adjoint's backward step.
+template <int P, typename R>
+__global__ void __launch_bounds__(256)
+k_keep_colliders(const R *khat, int64_t ld, const uint32_t *queue, const uint32_t *qcount, R *save, uint32_t *save_queue,
+                 uint32_t *save_count)
+{
+    const uint32_t count = *qcount;
+    if (blockIdx.x == 0 && threadIdx.x == 0) *save_count = count;
+    for (uint32_t j = blockIdx.x * blockDim.x + threadIdx.x; j < count; j += gridDim.x * blockDim.x) {
+        const uint32_t i = queue[j];
+        save_queue[j] = i;
+        if (!save) continue;
+#pragma unroll 6
+        for (int h = 0; h < 2 * P; ++h) save[(int64_t)h * ld + j] = khat[(int64_t)h * ld + i];
+    }
+}
+
 // Phase 2 of one block, block bid of the nb blocks doing phase 2 (any block size that is a
 // multiple of the group size).
 template <int P, int Q, typename R, bool EXT>

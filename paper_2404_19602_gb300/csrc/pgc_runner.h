@@ -80,6 +80,12 @@ public:
     // time step number `step` as two launches on one stream; if ev is non-NULL, ev[0..3] are
     // recorded before phase 1, after it, before phase 2 and after it
     virtual cudaError_t step(int64_t step, bool out_step, cudaStream_t s, cudaEvent_t *ev = nullptr) = 0;
+    // the adjoint's replay of step n: the two launches with f^n read from Hcur and f^{n+1} counted into Hnext
+    // (zeroed by the caller), the queued particles marked in `mark` (zeroed by the caller) and, if save
+    // is non-NULL, their queue kept in save_queue with its length in save_count and their drifted
+    // coefficients in save, [2P][ld], column j for queue entry j
+    virtual cudaError_t step_replay(int64_t n, const uint32_t *Hcur, uint32_t *Hnext, uint32_t *mark, void *save,
+                                    uint32_t *save_queue, uint32_t *save_count, cudaStream_t s) = 0;
     // the two launches of a step separately (phase 1 with a static tile assignment)
     virtual cudaError_t phase1(int64_t n, bool out_step, cudaStream_t s) = 0;
     virtual cudaError_t phase2(int64_t n, bool out_step, cudaStream_t s) = 0;

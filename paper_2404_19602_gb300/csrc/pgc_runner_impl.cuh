@@ -318,6 +318,23 @@ public:
         return e;
     }
 
+    cudaError_t step_replay(int64_t n, const uint32_t *Hcur, uint32_t *Hnext, uint32_t *mark, void *save,
+                            uint32_t *save_queue, uint32_t *save_count, cudaStream_t s) override
+    {
+        StepArgs<P, Q, R> a = args_at(n);
+        a.Hcur = Hcur;
+        a.Hnext = Hnext;
+        a.Hclear = Hnext;
+        a.hist_elems = 0;   // nothing to clear
+        a.mark = mark;
+        a.mark_clear = nullptr;
+        k_phase1<P, Q, R><<<grid1_, P1Threads<P, Q, R>::value, win_bytes_, s>>>(a);
+        k_keep_colliders<P, R><<<num_sms_, 256, 0, s>>>(a.khat, a.ld, a.queue, a.qcount, static_cast<R *>(save), save_queue, save_count);
+        k_phase2<P, Q, R, false><<<grid2_, kPhase2Threads, 0, s>>>(a);
+        count_launch(3);
+        return cudaGetLastError();
+    }
+
     cudaError_t hist_at(const double *psi, double xs, uint32_t *out, cudaStream_t s) override
     {
         ReconArgs<P, Q, R> z;
