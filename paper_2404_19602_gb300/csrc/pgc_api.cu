@@ -408,30 +408,29 @@ struct ObsFin {
     int nz, g;
 };
 
-// Thread t sums column t % 96 over the rows congruent to t / 96 modulo kObsFinSlots, then the slots in
-// order (one thread per column took 26 us for 304 rows, a chain of FP64 adds; 20 us for 608 now).
-constexpr int kObsFinSlots = 8;
-__global__ void __launch_bounds__(kObsZ * 3 * kObsFinSlots)
+// Block z reduces the three columns of point z: 64 threads a column sum every 64th row, then a tree (one
+// block for all columns, eight threads each, took 20 us for 608 rows: a chain of FP64 adds behind
+// memory latency; 26 us at 304 rows with one thread each; 4 us).
+constexpr int kObsFinRows = 64;
+__global__ void __launch_bounds__(3 * kObsFinRows)
 k_obs_fin(const double *part, const __grid_constant__ ObsFin f, double *out)
 {
-    __shared__ double S[kObsFinSlots][kObsZ * 3];
-    const int t = threadIdx.x, col = t % (kObsZ * 3), slot = t / (kObsZ * 3);
-    S[slot][col] = strided_sum(part, slot, f.g, kObsFinSlots, kObsZ * 3, col, 0.0);
+    __shared__ double S[3][kObsFinRows];
+    const int z = blockIdx.x, c = threadIdx.x / kObsFinRows, r = threadIdx.x % kObsFinRows;
+    S[c][r] = strided_sum(part, r, f.g, kObsFinRows, kObsZ * 3, z * 3 + c, 0.0);
     __syncthreads();
-    if (slot == 0) {
-        double s = 0.0;
 #pragma unroll
-        for (int k = 0; k < kObsFinSlots; ++k) s += S[k][col];
-        S[0][col] = s;
+    for (int w = kObsFinRows / 2; w > 0; w >>= 1) {
+        if (r < w) S[c][r] += S[c][r + w];
+        __syncthreads();
     }
-    __syncthreads();
-    if (t < f.nz) {
+    if (threadIdx.x == 0) {
         const double qe = 1.602176634e-19;
-        const double vx = S[0][t * 3 + 0] * f.scale_v, vy = S[0][t * 3 + 1] * f.scale_v;
-        out[t * 4 + 0] = vx;
-        out[t * 4 + 1] = vy;
-        out[t * 4 + 2] = S[0][t * 3 + 2] * f.inv_N;
-        out[t * 4 + 3] = -qe * f.n[t] * vx;
+        const double vx = S[0][0] * f.scale_v, vy = S[1][0] * f.scale_v;
+        out[z * 4 + 0] = vx;
+        out[z * 4 + 1] = vy;
+        out[z * 4 + 2] = S[2][0] * f.inv_N;
+        out[z * 4 + 3] = -qe * f.n[z] * vx;
     }
 }
 
@@ -786,6 +785,12 @@ pgc_status pgc_init(const pgc_config *cfg, void *d_state, void *d_hist, void *d_
     // collider work is itself throughput-bound (many chains per lane group) and, fused, holds
     // most resident blocks for the whole launch: measured slower, so off by default there
     ctx->pipeline = (ctx->run->fused() && L.P * L.Q <= 64) ? 1 : 0;
+    // The larger one-dimensional shapes: two launches of one latency chain each at the sizes of the error
+    // study, so fused is faster up to 2e5 particles (us a step, two launches / fused: 21 nodes 32.3 /
+    // 26.2 at 1e4, 69.5 / 64.5 at 2e5, 227 / 236 at 1e6; 9 nodes 23.6 / 17.6, 41.1 / 34.3, 108 / 113).  Only
+    // for calls without moment records: the states are the same bit for bit, the records' FP32 warp
+    // sums are grouped differently.
+    ctx->pipeline_auto = (!ctx->pipeline && ctx->run->fused() && L.d == 1 && cfg->precision == PGC_FP32 && cfg->n_particles <= 200000) ? 1 : 0;
     if (cfg->tc_proj != PGC_TC_OFF) {
         if ((e = ctx->run->set_tc(cfg->tc_proj)) != cudaSuccess) {
             delete ctx->run; delete ctx;
@@ -915,7 +920,8 @@ pgc_status pgc_step(pgc_ctx *ctx, int64_t n_steps, int32_t moments_every)
         pending[sl] = false;
         return cudaStreamWaitEvent(s, ctx->fin_done[sl], 0);
     };
-    if (e == cudaSuccess && (!ctx->pipeline || n_steps < 2)) {
+    const bool pipelined = n_steps >= 2 && (ctx->pipeline || (ctx->pipeline_auto && moments_every <= 0));
+    if (e == cudaSuccess && !pipelined) {
         for (int64_t k = 0; k < n_steps && e == cudaSuccess; ++k) {
             const int64_t n = n0 + k;
             hist_max(n);
@@ -971,6 +977,7 @@ pgc_status pgc_set_pipeline(pgc_ctx *ctx, int32_t on)
     if (on != 0 && on != 1) return fail(ctx, PGC_EINVAL, "on must be 0 or 1");
     if (on && !ctx->run->fused()) return fail(ctx, PGC_EUNSUPPORTED, "no pipelined step kernel for this shape (P * Q > 64)");
     ctx->pipeline = on;
+    ctx->pipeline_auto = 0;
     return PGC_OK;
 }
 
@@ -1177,7 +1184,7 @@ pgc_status pgc_observe_at(pgc_ctx *ctx, const double *h_z, int32_t nz, double *h
             f.inv_N = 1.0 / (double)ctx->b.N;
             f.nz = nzc;
             f.g = g;
-            k_obs_fin<<<1, kObsZ * 3 * kObsFinSlots, 0, ctx->stream>>>(ctx->obs_part, f, ctx->obs_out + (size_t)(j0 - out0) * 4);
+            k_obs_fin<<<nzc, 3 * kObsFinRows, 0, ctx->stream>>>(ctx->obs_part, f, ctx->obs_out + (size_t)(j0 - out0) * 4);
             count_launch();
             e = cudaGetLastError();
         }

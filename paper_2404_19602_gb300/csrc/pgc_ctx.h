@@ -31,6 +31,7 @@ struct pgc_ctx {
     bool sampled = false;  // state comes from the initial Fermi-Dirac sampling (no upload since)
     std::string err;
     int pipeline = 1;  // pipelined (fused) form of multi-step pgc_step calls (pgc_set_pipeline)
+    int pipeline_auto = 0;  // calls without moment records take the pipelined form (see pgc_init)
     // kernel timing samples (pgc_profile): events around phase 1 / phase 2 of sampled steps
     int prof_every = 0;
     std::vector<cudaEvent_t> prof_ev;  // 4 per sample
