@@ -83,7 +83,7 @@ k_phase1_batch(const __grid_constant__ BatchArgs<P, Q, R> a)
     __shared__ typename MomAcc<R>::T smom[NW][Q * 3];
     __shared__ int64_t stile[kBatchMaxCases + 1];
     __shared__ __align__(16) uint32_t snd[(sizeof(Nodes<P, Q, R>) + 3) / 4];
-    __shared__ uint32_t s_aside[NW][AsideList<PPT>::cap];
+    __shared__ uint32_t s_aside[NW][AsideList<PPT>::cap], s_qlist[NW][AsideList<PPT>::cap], s_qbase[NW + 1];
     extern __shared__ __align__(16) uint32_t swin[];
     const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
     const int64_t step = *a.d_step;
@@ -94,7 +94,7 @@ k_phase1_batch(const __grid_constant__ BatchArgs<P, Q, R> a)
     __syncthreads();
     const int64_t NN = (int64_t)a.ph.Nk * a.ph.Nk;
     const int64_t helems = (int64_t)Q * NN;
-    int cur = -1, n_aside = 0;
+    int cur = -1, n_aside = 0, n_q = 0;
     uint32_t *aside = s_aside[warp];
     unsigned int oog = 0u;
     for (int64_t tile = blockIdx.x; tile < a.ntiles; tile += gridDim.x) {
@@ -130,7 +130,7 @@ k_phase1_batch(const __grid_constant__ BatchArgs<P, Q, R> a)
         const int64_t p1 = min(cd.N, p0 + a.tile);
         for (int64_t base = p0; base < p1; base += (int64_t)blockDim.x * PPT)
             phase1_pass<P, Q, R, HistWin<P, Q, R>::batchW, PPT>(a.ph, nd, t, base + (int64_t)threadIdx.x * PPT, swin, a.win_r0, a.use_win != 0, a.kk_in,
-                                      out, smom[warp], aside, n_aside, oog);
+                                      out, smom[warp], aside, n_aside, s_qlist[warp], n_q, oog);
         if (n_aside > 0) {
             count_aside<P, Q, R, HistWin<P, Q, R>::batchW>(a.ph, nd, t, aside, n_aside, swin, a.win_r0, a.use_win != 0, oog);
             n_aside = 0;
@@ -147,6 +147,7 @@ k_phase1_batch(const __grid_constant__ BatchArgs<P, Q, R> a)
         if (lane == 0 && oog) atomicAdd(&cd.counters[4], (unsigned long long)oog);
         oog = 0u;
     }
+    queue_block(a.qcount + (step & 1), a.queue, s_qlist[warp], n_q, s_qbase);
 }
 
 template <int P, int Q, typename R>

@@ -638,6 +638,35 @@ struct P1Target {
 // are taken 32 at a time (at most 31 stay between passes).
 template <int PPT> struct AsideList { static constexpr int cap = 32 * (PPT + 1); };
 
+// The colliders a warp finds wait in a list of their own (also AsideList::cap entries) and reach the
+// queue 32 at a time, the rest of a block's warps together at its end: every append is an atomic with
+// a result on one address of the launch, which L2 serves about every 2 ns.  One per warp pass with a
+// collider (a quarter of them) was the kernel's time in the small shapes: 64 cases of 5e4 particles,
+// one node, 25000 appends a step, 50 -> 41.5 us.
+__device__ __forceinline__ void queue_warp(uint32_t *qcount, uint32_t *queue, const uint32_t *list, int lane)
+{
+    __syncwarp();
+    uint32_t pos = 0;
+    if (lane == 0) pos = atomicAdd(qcount, 32u);
+    pos = __shfl_sync(0xffffffffu, pos, 0);
+    queue[pos + lane] = list[lane];
+    __syncwarp();
+}
+// The remainders (n < 32 each) of a block's warps; s_base: nwarps + 1 words.  Synchronises the block.
+__device__ __forceinline__ void queue_block(uint32_t *qcount, uint32_t *queue, const uint32_t *list, int n, uint32_t *s_base)
+{
+    const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5, nw = blockDim.x >> 5;
+    if (lane == 0) s_base[warp] = (uint32_t)n;
+    __syncthreads();
+    if (threadIdx.x == 0) {
+        uint32_t s = 0;
+        for (int v = 0; v < nw; ++v) { const uint32_t c = s_base[v]; s_base[v] = s; s += c; }
+        s_base[nw] = s ? atomicAdd(qcount, s) : 0u;
+    }
+    __syncthreads();
+    if (lane < n) queue[s_base[nw] + s_base[warp] + lane] = list[lane];
+}
+
 // Counts the histogram cells of n <= 32 such particles (one per lane) from their stored state.
 template <int P, int Q, typename R, int W>
 __device__ __forceinline__ void count_aside(const Phys<R> &ph, const Nodes<P, Q, R> &nd, const P1Target<R> &t, const uint32_t *list,
@@ -674,7 +703,8 @@ template <int P, int Q, typename R, int W = HistWin<P, Q, R>::W, int PPT = Phase
 __device__ __forceinline__ void phase1_pass(const Phys<R> &ph, const Nodes<P, Q, R> &nd, const P1Target<R> &t,
                                             int64_t i0, uint32_t *swin, int win_r0, bool use_win, float kk_in, bool out_step,
                                             typename MomAcc<R>::T *smom_warp, uint32_t *aside, int &n_aside,
-                                            unsigned int &oog, const unsigned long long *spsi = nullptr)
+                                            uint32_t *qlist, int &n_q, unsigned int &oog,
+                                            const unsigned long long *spsi = nullptr)
 {
     const int lane = threadIdx.x & 31;
     const int64_t NN = (int64_t)ph.Nk * ph.Nk;
@@ -787,18 +817,19 @@ __device__ __forceinline__ void phase1_pass(const Phys<R> &ph, const Nodes<P, Q,
                 n_aside += __popc(am);
             }
         }
-        // colliders go to the queue (warp-aggregated append)
+        // colliders go to the warp's list for the queue
         const unsigned int mask = __ballot_sync(0xffffffffu, maybe);
         if (mask) {
-            const int leader = __ffs(mask) - 1;
-            uint32_t basepos = 0;
-            if (lane == leader) basepos = atomicAdd(t.qcount, (uint32_t)__popc(mask));
-            basepos = __shfl_sync(0xffffffffu, basepos, leader);
             if (maybe) {
-                t.queue[basepos + __popc(mask & ((1u << lane) - 1u))] = t.qoffset + (uint32_t)i;
+                qlist[n_q + __popc(mask & ((1u << lane) - 1u))] = t.qoffset + (uint32_t)i;
                 if (t.mark) atomicOr(&t.mark[i >> 5], 1u << (i & 31));
             }
+            n_q += __popc(mask);
         }
+    }
+    while (n_q >= 32) {
+        n_q -= 32;
+        queue_warp(t.qcount, t.queue, qlist + n_q, lane);
     }
     if (out_step) {
         if constexpr (TensorShape<P, Q>::value && sizeof(R) == 4 && PPT == 1) {
@@ -921,8 +952,9 @@ __device__ __forceinline__ void phase1_block(const StepArgs<P, Q, R> &a, int bid
     __shared__ uint32_t s_tile;
     __shared__ uint32_t s_aside[NW][AsideList<PPT>::cap];
     const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
-    uint32_t *aside = s_aside[warp];
-    int n_aside = 0;
+    __shared__ uint32_t s_qlist[NW][AsideList<PPT>::cap], s_qbase[NW + 1];
+    uint32_t *aside = s_aside[warp], *qlist = s_qlist[warp];
+    int n_aside = 0, n_q = 0;
     using SP = StagePsi<P, Q, R>;
     __shared__ __align__(16) unsigned long long spsi[SP::elems];
     if constexpr (SP::value)
@@ -985,20 +1017,20 @@ __device__ __forceinline__ void phase1_block(const StepArgs<P, Q, R> &a, int bid
             if (tl >= ntiles) break;
             guard_window();
             phase1_pass<P, Q, R>(a.ph, a.nd, t, tl * tile + (int64_t)threadIdx.x * PPT, swin, a.win_r0,
-                                 a.use_win != 0, a.kk_in, a.out_step != 0, smom[warp], aside, n_aside, oog, spsi);
+                                 a.use_win != 0, a.kk_in, a.out_step != 0, smom[warp], aside, n_aside, qlist, n_q, oog, spsi);
         }
     } else {
         for (int64_t base = (int64_t)bid * tile; base < a.N; base += (int64_t)nb * tile) {
             guard_window();
             phase1_pass<P, Q, R>(a.ph, a.nd, t, base + (int64_t)threadIdx.x * PPT, swin, a.win_r0, a.use_win != 0, a.kk_in,
-                                 a.out_step != 0, smom[warp], aside, n_aside, oog, spsi);
+                                 a.out_step != 0, smom[warp], aside, n_aside, qlist, n_q, oog, spsi);
         }
     }
     if (n_aside > 0)
         count_aside<P, Q, R, HistWin<P, Q, R>::W>(a.ph, a.nd, t, aside, n_aside, swin, a.win_r0, a.use_win != 0, oog);
     oog = warp_sum(oog);
     if (lane == 0 && oog) atomicAdd(&a.counters[4], (unsigned long long)oog);
-    __syncthreads();
+    queue_block(t.qcount, t.queue, qlist, n_q, s_qbase);   // (synchronises)
     if (a.use_win) flush_window<Q, HistWin<P, Q, R>::W>(swin, a.Hnext, a.ph.Nk, a.win_r0);
     if (a.out_step) {
         for (int j = threadIdx.x; j < Q * 3; j += blockDim.x) {
