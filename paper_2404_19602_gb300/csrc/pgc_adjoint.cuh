@@ -558,6 +558,7 @@ k_adj_collide(const __grid_constant__ AdjArgs<P, Q, R> a)
 // ------------------------------------------------------------------------------------------
 template <int P, int Q>
 struct AdjInitArgs {
+    int32_t ng;                      // distinct band minima (see InitArgs; nodes of one share d eps0 / d theta)
     double wpsi[Q * P];
     double eps0[Q];
     double de0[Q][NTH];
@@ -584,7 +585,7 @@ k_adj_init(const __grid_constant__ AdjArgs<P, Q, R> a, const __grid_constant__ A
             lx[h] = (double)a.lam[(int64_t)h * a.ld + i];
             ly[h] = (double)a.lam[(int64_t)(P + h) * a.ld + i];
         }
-        for (int q = 0; q < Q; ++q) {
+        for (int q = 0; q < ia.ng; ++q) {
             // d|k|/d eps0 with deps/deps0 = rho(eps0)(1-u)/rho(eps), rho(e) = e / (1 + exp((e-mu)/kT))
             const double e0 = ia.eps0[q];
             double dkm;
@@ -678,18 +679,17 @@ public:
                 if (std::fabs(a_.ddhat[k][h]) <= 1e-13 * ddmax) a_.ddhat[k][h] = 0.0;
                 if (a_.ddhat[k][h] != 0.0) a_.ddmask |= 1u << h;
             }
-        for (int i = 0; i < Q * P; ++i) ia_.wpsi[i] = t.wpsi[i];
-        for (int q = 0; q < Q; ++q) {
-            ia_.eps0[q] = t.eps0[q];
-            for (int k = 0; k < NTH; ++k) ia_.de0[q][k] = a_.de0[q][k];
-        }
+        int of[Q];
+        ia_.ng = fd_groups(t.eps0.data(), Q, t.wpsi.data(), P, ia_.eps0, ia_.wpsi, of);
+        for (int q = 0; q < Q; ++q)
+            for (int k = 0; k < NTH; ++k) ia_.de0[of[q]][k] = a_.de0[q][k];
         ia_.mu = t.mu;
         ia_.kT = t.kT;
         ia_.hvF = t.hvF;
         if (b.fdtab) {   // written by the sampling of the context (the adjoint starts from its sampled state)
-            ia_.fd = fd_plan(ia_.eps0, Q, t.mu, t.kT, ia_.ratio);
+            ia_.fd = fd_plan(ia_.eps0, ia_.ng, t.mu, t.kT, ia_.ratio);
             if (ia_.fd.n > 0) ia_.fd.tab = b.fdtab;
-            for (int q = 0; q < Q; ++q) {
+            for (int q = 0; q < ia_.ng; ++q) {
                 const double w0 = ia_.eps0[q] / t.kT;
                 ia_.y0[q] = w0 * w0;
                 ia_.ie0[q] = 1.0 / (1.0 + std::exp(w0 - ia_.fd.m));

@@ -184,6 +184,24 @@ inline long double fd_G_host(long double w, long double m)
     return b >= 0.0L ? w * l + li : w * l - b * (m + 0.5L * b) + pi * pi / 6.0L - li;
 }
 
+// Groups the nodes by band minimum: eg[0..ng) the distinct ones in order of first appearance, of[q] the
+// group of node q, wg[g][h] the weights w[q][h] summed over the group's nodes.
+inline int fd_groups(const double *eps0, int Q, const double *w, int P, double *eg, double *wg, int *of)
+{
+    int ng = 0;
+    for (int q = 0; q < Q; ++q) {
+        int g = 0;
+        while (g < ng && eg[g] != eps0[q]) ++g;
+        if (g == ng) {
+            eg[ng++] = eps0[q];
+            for (int h = 0; h < P; ++h) wg[g * P + h] = 0.0;
+        }
+        of[q] = g;
+        for (int h = 0; h < P; ++h) wg[g * P + h] += w[q * P + h];
+    }
+    return ng;
+}
+
 // The table's layout for band minima eps0[0..Q); ratio[q] = G(w0_q) / Gmax.  Leaves tab null (no
 // table) when the range of r over the nodes needs more intervals than there is room for.
 inline FdInv fd_plan(const double *eps0, int Q, double mu, double kT, double *ratio)

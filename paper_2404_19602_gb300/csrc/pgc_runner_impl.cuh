@@ -84,8 +84,8 @@ public:
         args_.key0 = b.key0;
         args_.key1 = b.key1;
         args_.stream_id = b.stream_id;
-        for (int i = 0; i < Q * P; ++i) init_.wpsi[i] = t.wpsi[i];
-        for (int q = 0; q < Q; ++q) init_.eps0[q] = t.eps0[q];
+        int of[Q];
+        init_.ng = fd_groups(t.eps0.data(), Q, t.wpsi.data(), P, init_.eps0, init_.wpsi, of);
         init_.mu = t.mu;
         init_.kT = t.kT;
         init_.hvF = t.hvF;
@@ -103,7 +103,8 @@ public:
         win_bytes_ = HistWin<P, Q, R>::bytes;
         args_.win_r0 = window_r0(t.Nk, W);
         bool win = t.Nk >= W;
-        if (win && (cudaFuncSetAttribute(k_phase1<P, Q, R>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)win_bytes_) != cudaSuccess ||
+        if (win && (cudaFuncSetAttribute(k_observe<P, Q, R>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)win_bytes_) != cudaSuccess ||
+                    cudaFuncSetAttribute(k_phase1<P, Q, R>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)win_bytes_) != cudaSuccess ||
                     !fused_attr())) {
             cudaGetLastError();
             win = false;
@@ -132,8 +133,8 @@ public:
     cudaError_t init_sample(cudaStream_t s) override
     {
         if (b_.fdtab) {
-            init_.fd = fd_plan(init_.eps0, Q, init_.mu, init_.kT, init_.ratio);
-            for (int q = 0; q < Q; ++q) { const double w0 = init_.eps0[q] / init_.kT; init_.y0[q] = w0 * w0; }
+            init_.fd = fd_plan(init_.eps0, init_.ng, init_.mu, init_.kT, init_.ratio);
+            for (int q = 0; q < init_.ng; ++q) { const double w0 = init_.eps0[q] / init_.kT; init_.y0[q] = w0 * w0; }
             if (init_.fd.n > 0) {
                 k_fd_table<<<(init_.fd.n + 31) / 32, 32, 0, s>>>(init_.fd, b_.fdtab);
                 count_launch();
@@ -151,7 +152,7 @@ public:
         StepArgs<P, Q, R> a = args_;
         a.Hnext = b_.hist + (int64_t)buf * b_.hist_stride;
         a.out_step = 1;
-        k_observe<P, Q, R><<<grid1_, P1Threads<P, Q, R>::value, 0, s>>>(a);
+        launch_observe(a, s);
         count_launch();
         return cudaGetLastError();
     }
@@ -162,7 +163,7 @@ public:
         a.Hnext = hist;
         a.part1 = part;
         a.out_step = 1;
-        k_observe<P, Q, R><<<grid1_, P1Threads<P, Q, R>::value, 0, s>>>(a);
+        launch_observe(a, s);
         count_launch();
         return cudaGetLastError();
     }
@@ -369,6 +370,14 @@ public:
     }
 
 private:
+    // (the window of k_observe is the streaming kernel's; a tensor-core context counts without one here,
+    // its own has another layout)
+    void launch_observe(StepArgs<P, Q, R> &a, cudaStream_t s)
+    {
+        if (tc_mode_) a.use_win = 0;
+        k_observe<P, Q, R><<<grid1_, P1Threads<P, Q, R>::value, a.use_win ? win_bytes_ : 0, s>>>(a);
+    }
+
     void fill_phys(const HostTables &t)
     {
         Phys<R> &p = args_.ph;
