@@ -41,6 +41,7 @@ struct CaseDev {
 template <int P, int Q, typename R>
 struct BatchArgs {
     Phys<R> ph;
+    Nodes<P, Q, R> nd;         // of case 0: the basis tables and grid offsets, common to the cases
     CaseDev<P, Q, R> *cases;
     const int64_t *tile0s;     // [ncases + 1] tile prefix
     const int64_t *bases;      // [ncases + 1] particle prefix
@@ -74,9 +75,12 @@ __device__ __forceinline__ int find_case(const int64_t *prefix, int n, int64_t x
 // (four, two or one for the small bases; one for P = 21).
 template <int P> struct BatchPPTs { static constexpr int n = (P <= 8) ? 3 : 1; static constexpr int v[3] = {Phase1PPT<P>::value, 2, 1}; };
 
-// Any block size up to kPhase1Threads that is a multiple of 32 (the autotuner uses 128 and 256).
+// Any block size up to kPhase1Threads that is a multiple of 32 (the autotuner uses 128 and 256).  The
+// basis tables, common to the cases, are read from the parameter bank as the standalone kernel reads
+// them; from a staged copy every weight was a shared-memory load (835 warp instructions per 32
+// particles x 6 nodes against 477, 32 cases of 1.3e7 particles 245 -> 209 us a launch).
 template <int P, int Q, typename R, int PPT>
-__global__ void __launch_bounds__(kPhase1Threads)
+__global__ void __launch_bounds__(kPhase1Threads, P * Q <= 64 && sizeof(R) == 4 ? 3 : 1)
 k_phase1_batch(const __grid_constant__ BatchArgs<P, Q, R> a)
 {
     constexpr int NW = kPhase1Threads / 32;
@@ -128,11 +132,17 @@ k_phase1_batch(const __grid_constant__ BatchArgs<P, Q, R> a)
         t.key0 = cd.key0; t.key1 = cd.key1; t.stream_id = cd.stream_id; t.step = (uint32_t)step;
         const int64_t p0 = (tile - cd.tile0) * a.tile;
         const int64_t p1 = min(cd.N, p0 + a.tile);
-        for (int64_t base = p0; base < p1; base += (int64_t)blockDim.x * PPT)
-            phase1_pass<P, Q, R, HistWin<P, Q, R>::batchW, PPT>(a.ph, nd, t, base + (int64_t)threadIdx.x * PPT, swin, a.win_r0, a.use_win != 0, a.kk_in,
-                                      out, smom[warp], aside, n_aside, s_qlist[warp], n_q, oog);
+        for (int64_t base = p0; base < p1; base += (int64_t)blockDim.x * PPT) {
+            if (PPT == 1 || P > 1 || sizeof(R) == 8 || out) {
+                phase1_pass<P, Q, R, HistWin<P, Q, R>::batchW, PPT>(a.ph, a.nd, nd, t, base + (int64_t)threadIdx.x * PPT, swin, a.win_r0,
+                                                                    a.use_win != 0, a.kk_in, out, smom[warp], aside, n_aside, s_qlist[warp], n_q, oog);
+            } else {   // as in phase1_block
+                phase1_rolled<P, Q, R, HistWin<P, Q, R>::batchW, PPT>(a.ph, a.nd, nd, t, base, swin, a.win_r0, a.use_win != 0, a.kk_in,
+                                                                      smom[warp], aside, n_aside, s_qlist[warp], n_q, oog);
+            }
+        }
         if (n_aside > 0) {
-            count_aside<P, Q, R, HistWin<P, Q, R>::batchW>(a.ph, nd, t, aside, n_aside, swin, a.win_r0, a.use_win != 0, oog);
+            count_aside<P, Q, R, HistWin<P, Q, R>::batchW>(a.ph, a.nd, t, aside, n_aside, swin, a.win_r0, a.use_win != 0, oog);
             n_aside = 0;
         }
         __syncthreads();
@@ -322,6 +332,7 @@ public:
         // physics shared by all cases: take it from a single-case runner's argument block
         RunnerT<P, Q, R> proto(t0, cases[0].b, num_sms);
         a_.ph = proto.args().ph;
+        a_.nd = proto.args().nd;
         a_.cases = static_cast<CaseDev<P, Q, R> *>(sc.cases);
         a_.tile0s = sc.tile0s;
         a_.bases = sc.bases;

@@ -698,13 +698,15 @@ __device__ __forceinline__ void count_aside(const Phys<R> &ph, const Nodes<P, Q,
 
 // One pass of a block over blockDim * PPT consecutive particles starting at i0 + threadIdx*PPT:
 // drift, reconstruction, flight-time screen, histogram (window or global), queue, moments.
-// (PPT particles per thread; i0 a multiple of PPT.)
+// (PPT particles per thread; i0 a multiple of PPT.)  ndb: the basis and the grid offsets, nd: what
+// depends on the inputs (drift, band minima); a batch's cases share the former, which then stays in the
+// parameter bank.
 template <int P, int Q, typename R, int W = HistWin<P, Q, R>::W, int PPT = Phase1PPT<P>::value>
-__device__ __forceinline__ void phase1_pass(const Phys<R> &ph, const Nodes<P, Q, R> &nd, const P1Target<R> &t,
+__device__ __forceinline__ void phase1_pass(const Phys<R> &ph, const Nodes<P, Q, R> &ndb, const Nodes<P, Q, R> &nd, const P1Target<R> &t,
                                             int64_t i0, uint32_t *swin, int win_r0, bool use_win, float kk_in, bool out_step,
                                             typename MomAcc<R>::T *smom_warp, uint32_t *aside, int &n_aside,
                                             uint32_t *qlist, int &n_q, unsigned int &oog,
-                                            const unsigned long long *spsi = nullptr)
+                                            const unsigned long long *spsi = nullptr, const R *pre = nullptr)
 {
     const int lane = threadIdx.x & 31;
     const int64_t NN = (int64_t)ph.Nk * ph.Nk;
@@ -714,6 +716,10 @@ __device__ __forceinline__ void phase1_pass(const Phys<R> &ph, const Nodes<P, Q,
     // i0 is a multiple of PPT, so its PPT bits lie in one word
     const uint32_t skipbits = (t.skip && any) ? (t.skip[i0 >> 5] >> (i0 & 31)) & ((1u << PPT) - 1u) : 0u;
     if (any) {
+        if (PPT == 1 && pre) {   // loaded by the caller
+#pragma unroll
+            for (int h = 0; h < P; ++h) { cx[0][h] = pre[h]; cy[0][h] = pre[P + h]; }
+        } else
 #pragma unroll
         for (int h = 0; h < P; ++h) {
             R vx[PPT], vy[PPT];
@@ -766,14 +772,14 @@ __device__ __forceinline__ void phase1_pass(const Phys<R> &ph, const Nodes<P, Q,
                         for (int h = 0; h < P; ++h) s2 = f2_fma(f2_pack(cx[e][h], cy[e][h]), (h & 1) ? w[h >> 1].y : w[h >> 1].x, s2);
                         float kx, ky;
                         f2_unpack(s2, kx, ky);
-                        cell[q] = window_code<W>(kx, ky, nd.lk2[q], inv2, magic2);
+                        cell[q] = window_code<W>(kx, ky, ndb.lk2[q], inv2, magic2);
                         const float kk = knorm2(kx, ky);
                         km.m = fmaxf(km.m, kk);
                         km.n = max3_nan(km.n, kk, kk);
                     }
                 } else {
-                    recon_all(nd, cx[e], cy[e], [&](int q, R kx, R ky) {
-                        cell[q] = window_code<W>(kx, ky, nd.lk2[q], inv2, magic2);
+                    recon_all(ndb, cx[e], cy[e], [&](int q, R kx, R ky) {
+                        cell[q] = window_code<W>(kx, ky, ndb.lk2[q], inv2, magic2);
                         km.add(q, Q, knorm2(kx, ky));
                     });
                 }
@@ -784,8 +790,8 @@ __device__ __forceinline__ void phase1_pass(const Phys<R> &ph, const Nodes<P, Q,
                 // instruction per 16 clocks; the reconstruction is what it has to do), else in FP64
                 KkMax km;
                 float edge = 1.0f;
-                recon_all(nd, cx[e], cy[e], [&](int q, R kx, R ky) {
-                    cell[q] = window_code_f64<W>(kx, ky, nd.lk2[q], inv2, win_r0, edge);
+                recon_all(ndb, cx[e], cy[e], [&](int q, R kx, R ky) {
+                    cell[q] = window_code_f64<W>(kx, ky, ndb.lk2[q], inv2, win_r0, edge);
                     const float xf = (float)kx, yf = (float)ky;
                     km.add(q, Q, xf * xf + yf * yf);
                 });
@@ -793,7 +799,7 @@ __device__ __forceinline__ void phase1_pass(const Phys<R> &ph, const Nodes<P, Q,
                 maybe = sc > 0;
                 if (sc < 0) {
                     R kk = (R)0;
-                    recon_all_rolled(nd, cx[e], cy[e], [&](int, R kx, R ky) { kk = fmax(kk, knorm2(kx, ky)); });
+                    recon_all_rolled(ndb, cx[e], cy[e], [&](int, R kx, R ky) { kk = fmax(kk, knorm2(kx, ky)); });
                     maybe = screen_maybe(ph, nd, kk, r.x);
                 }
                 in_window = km.n <= kk_in && edge > kCellGuard * (float)ph.Nk;
@@ -838,7 +844,7 @@ __device__ __forceinline__ void phase1_pass(const Phys<R> &ph, const Nodes<P, Q,
             // quantity j is value 3 q + j)
             float buf[16];
             const bool fin = finished[0];
-            recon_all(nd, cx[0], cy[0], [&](int q, R kx, R ky) {
+            recon_all(ndb, cx[0], cy[0], [&](int q, R kx, R ky) {
                 float o[3] = {0.0f, 0.0f, 0.0f};
                 if (fin) observe_fast(ph, kx - nd.xs[q], ky, nd.eps0[q], o[0], o[1], o[2]);
 #pragma unroll
@@ -861,7 +867,7 @@ __device__ __forceinline__ void phase1_pass(const Phys<R> &ph, const Nodes<P, Q,
                 for (int e = 0; e < PPT; ++e)
                     if (finished[e]) {
                         float kx, ky, a1, a2, a3;
-                        recon_node(nd, q, cx[e], cy[e], kx, ky);
+                        recon_node(ndb, q, cx[e], cy[e], kx, ky);
                         observe(ph, kx - nd.xs[q], ky, nd.eps0[q], a1, a2, a3);
                         s[0] += a1; s[1] += a2; s[2] += a3;
                     }
@@ -875,7 +881,7 @@ __device__ __forceinline__ void phase1_pass(const Phys<R> &ph, const Nodes<P, Q,
                 for (int e = 0; e < PPT; ++e)
                     if (finished[e]) {
                         R kx, ky, a1, a2, a3;
-                        recon_node(nd, q, cx[e], cy[e], kx, ky);
+                        recon_node(ndb, q, cx[e], cy[e], kx, ky);
                         observe(ph, kx - nd.xs[q], ky, nd.eps0[q], a1, a2, a3);
                         vx += a1; vy += a2; en += a3;
                     }
@@ -892,7 +898,35 @@ __device__ __forceinline__ void phase1_pass(const Phys<R> &ph, const Nodes<P, Q,
     }
     while (n_aside >= 32) {
         n_aside -= 32;
-        count_aside<P, Q, R, W>(ph, nd, t, aside + n_aside, 32, swin, win_r0, use_win, oog);
+        count_aside<P, Q, R, W>(ph, ndb, t, aside + n_aside, 32, swin, win_r0, use_win, oog);
+    }
+}
+
+// PPT passes of one particle per thread over the PPT * blockDim particles from `base` (a step without
+// moments), each pass's coefficients loaded behind the one before it.
+template <int P, int Q, typename R, int W, int PPT>
+__device__ __forceinline__ void phase1_rolled(const Phys<R> &ph, const Nodes<P, Q, R> &ndb, const Nodes<P, Q, R> &nd, const P1Target<R> &t,
+                                              int64_t base, uint32_t *swin, int win_r0, bool use_win, float kk_in,
+                                              typename MomAcc<R>::T *smom_warp, uint32_t *aside, int &n_aside, uint32_t *qlist,
+                                              int &n_q, unsigned int &oog)
+{
+    R nx[2 * P];
+    auto load = [&](int64_t i) {
+        if (i < t.N) {
+#pragma unroll
+            for (int h = 0; h < 2 * P; ++h) nx[h] = t.khat[(int64_t)h * t.ld + i];
+        }
+    };
+    int64_t i = base + threadIdx.x;
+    load(i);
+#pragma unroll 1
+    for (int e = 0; e < PPT; ++e, i += blockDim.x) {
+        R c[2 * P];
+#pragma unroll
+        for (int h = 0; h < 2 * P; ++h) c[h] = nx[h];
+        if (e + 1 < PPT) load(i + blockDim.x);
+        phase1_pass<P, Q, R, W, 1>(ph, ndb, nd, t, i, swin, win_r0, use_win, kk_in, false, smom_warp, aside, n_aside, qlist, n_q, oog,
+                                   nullptr, c);
     }
 }
 
@@ -1007,6 +1041,19 @@ __device__ __forceinline__ void phase1_block(const StepArgs<P, Q, R> &a, int bid
         }
         since_flush += tile;
     };
+    // One node: a step without moments takes the tile's particles one per thread at a time (coalesced 4-byte
+    // loads, each pass's ahead of the one before).  64 cases of 5e4 particles: 41.5 -> 37.6 us a launch.  With
+    // 6 nodes the rolled form is slower (1e6 particles 26 -> 32 us: its loads are waited for one by one).
+    auto pass = [&](int64_t base) {
+        constexpr int W = HistWin<P, Q, R>::W;
+        if (PPT == 1 || P > 1 || sizeof(R) == 8 || a.out_step) {
+            phase1_pass<P, Q, R, W, PPT>(a.ph, a.nd, a.nd, t, base + (int64_t)threadIdx.x * PPT, swin, a.win_r0, a.use_win != 0, a.kk_in,
+                                         a.out_step != 0, smom[warp], aside, n_aside, qlist, n_q, oog, spsi);
+        } else {
+            phase1_rolled<P, Q, R, W, PPT>(a.ph, a.nd, a.nd, t, base, swin, a.win_r0, a.use_win != 0, a.kk_in, smom[warp], aside, n_aside,
+                                           qlist, n_q, oog);
+        }
+    };
     if (a.tilectr) {
         const int64_t ntiles = (a.N + tile - 1) / tile;
         for (;;) {
@@ -1016,14 +1063,12 @@ __device__ __forceinline__ void phase1_block(const StepArgs<P, Q, R> &a, int bid
             __syncthreads();   // every thread has read s_tile before it is overwritten
             if (tl >= ntiles) break;
             guard_window();
-            phase1_pass<P, Q, R>(a.ph, a.nd, t, tl * tile + (int64_t)threadIdx.x * PPT, swin, a.win_r0,
-                                 a.use_win != 0, a.kk_in, a.out_step != 0, smom[warp], aside, n_aside, qlist, n_q, oog, spsi);
+            pass(tl * tile);
         }
     } else {
         for (int64_t base = (int64_t)bid * tile; base < a.N; base += (int64_t)nb * tile) {
             guard_window();
-            phase1_pass<P, Q, R>(a.ph, a.nd, t, base + (int64_t)threadIdx.x * PPT, swin, a.win_r0, a.use_win != 0, a.kk_in,
-                                 a.out_step != 0, smom[warp], aside, n_aside, qlist, n_q, oog, spsi);
+            pass(base);
         }
     }
     if (n_aside > 0)
