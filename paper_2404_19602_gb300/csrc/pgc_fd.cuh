@@ -18,7 +18,8 @@
 // particle and node, where the iteration (fd_inverse) takes a 30-step FP32 bisection and about eight
 // FP64 evaluations of G (each an exp, two log1p, a division and a 12-term series).  The FP64 pipe of
 // this part issues two lanes per clock and SM, and bounds both.  Measured: the sampling of 500 000
-// particles at 36 nodes 208 -> 1.6 ms, of 1e6 particles at 6 nodes 56.2 -> 0.44 ms, its
+// particles at 36 nodes 208 -> 1.6 ms (0.35 ms over the distinct band minima, k_init), of 1e6
+// particles at 6 nodes 56.2 -> 0.44 ms, its
 // sensitivities at 5e5 x 6 nodes 32.2 -> 0.5 ms; the table itself takes 26 us (a warp per
 // block: latency of two FP64 Newton steps).  Error of eps against extended precision: rms
 // 3.9e-16 (iteration: 4.1e-16) for eps0 in [0.05, 0.15] eV at eps_F = 0.4 eV, 300 K.

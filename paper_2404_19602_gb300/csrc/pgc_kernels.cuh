@@ -11,15 +11,15 @@
 //       counter, so that no separate memset is needed.
 //   k_phase2 (queued particles only): the exact collision loop of Algorithm 1 / 2 with the
 //       Pauli test against f^n, then the histogram f^{n+1} and moments of the final state.
-// On moment steps a one-block k_finalize reduces the block partial sums in a fixed order and
-// writes the node values, mean and variance of the record (Sec. 4.2).
+// On moment steps k_finalize_cols reduces the block partial sums in a fixed order, one block per
+// column, and writes the node values, mean and variance of the record (Sec. 4.2).
 //
 // Pipelined form (several steps per call): k_phase2<EXT = true> of step n, after the collision
 // loop of a queued particle, carries that particle on through the drift and the flight-time
 // screen of step n + 1 (finishing it there, or queueing it for step n + 1), and k_phase1 of step
-// n + 1 skips the particles queued at step n (a bitmap).  The two kernels then touch disjoint
-// particles and buffers and run concurrently on two streams; every particle undergoes the same
-// arithmetic as in the two-launch form, so the trajectories are identical.
+// n + 1 skips the particles queued at step n (a bitmap).  The two then touch disjoint particles and
+// buffers and are the two roles of one launch, k_step; every particle undergoes the same arithmetic
+// as in the two-launch form, so the trajectories are identical.
 #pragma once
 
 #include "pgc_device.cuh"
@@ -1484,9 +1484,10 @@ __device__ __forceinline__ void collide_particle(const Phys<R> &ph, const Nodes<
 // and the warp runs their union.  A queue of at most half as many entries as warps is spread one group
 // per warp, over the blocks first: the chain of one particle is then the kernel's time
 // (deterministic FP64 run of 1e4 particles, ~90 colliders a step: 99.6 us a step in three warps
-// of one block, 77 us spread).  A longer one fills whole warps: spread, 6 nodes, 5e5 particles took 25.0
-// instead of 22.0 us a fused step (every collider block then holds its place on an SM) and 43.8
-// instead of 37.7 us in the adjoint's collider kernel.
+// of one block, 77 us spread; 32 us with the edge table and the root starts as well).  A longer one
+// fills whole warps: spread, 6 nodes, 5e5 particles took 25.0 instead of 22.0 us a fused step (every
+// collider block then holds its place on an SM) and 43.8 instead of 37.7 us in the adjoint's collider
+// kernel.
 struct QueueShare { uint32_t first, stride; };
 template <int G>
 __device__ __forceinline__ QueueShare queue_share(uint32_t count, int bid, int nb)
