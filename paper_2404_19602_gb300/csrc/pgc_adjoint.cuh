@@ -148,7 +148,9 @@ k_adj_screen(const __grid_constant__ AdjArgs<P, Q, R> a)
                     R kx, ky;
                     recon_node(nd, q, cx, cy, kx, ky);
                     const R e0 = nd.eps0[q], hv = ph.hvF;
-                    const R eps = rsqrt_<R>(ph.hvF2 * (kx * kx + ky * ky) + e0 * e0);
+                    // (which products are rounded is written out: left to the compiler it follows the surrounding
+                    // code, and moves an FP32 gradient by 1e-8)
+                    const R eps = rsqrt_<R>(fma(e0, e0, ph.hvF2 * fma(kx, kx, ky * ky)));
                     const R ie = (R)1 / eps, ie3 = ie * ie * ie;
                     const R vhat = hv * kx * ie;
                     const R dvx = hv * ie - hv * ph.hvF2 * kx * kx * ie3;
