@@ -77,8 +77,8 @@ template <int P> struct BatchPPTs { static constexpr int n = (P <= 8) ? 3 : 1; s
 
 // Any block size up to kPhase1Threads that is a multiple of 32 (the autotuner uses 128 and 256).  The
 // basis tables, common to the cases, are read from the parameter bank as the standalone kernel reads
-// them; from a staged copy every weight was a shared-memory load (835 warp instructions per 32
-// particles x 6 nodes against 477, 32 cases of 1.3e7 particles 245 -> 209 us a launch).
+// them; from a staged copy every weight was a shared-memory load (the LSU data path 47 % busy against
+// 15 %; 32 cases of 1.3e7 particles 245 -> 209 us a launch).
 template <int P, int Q, typename R, int PPT>
 __global__ void __launch_bounds__(kPhase1Threads, P * Q <= 64 && sizeof(R) == 4 ? 3 : 1)
 k_phase1_batch(const __grid_constant__ BatchArgs<P, Q, R> a)
