@@ -688,7 +688,7 @@ public:
         ia_.mu = t.mu;
         ia_.kT = t.kT;
         ia_.hvF = t.hvF;
-        if (b.fdtab) {   // written by the sampling of the context (the adjoint starts from its sampled state)
+        if (b.fdtab && !FdPerNode<Q, R>::value(ia_.ng)) {   // written by the sampling of the context (the adjoint starts from its sampled state)
             ia_.fd = fd_plan(ia_.eps0, ia_.ng, t.mu, t.kT, ia_.ratio);
             if (ia_.fd.n > 0) ia_.fd.tab = b.fdtab;
             for (int q = 0; q < ia_.ng; ++q) {

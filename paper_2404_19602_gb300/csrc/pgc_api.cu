@@ -715,8 +715,13 @@ static pgc_status observe_current(pgc_ctx *ctx, bool record, bool set_nmax)
         f.g1 = ctx->run->grid1();
         f.g2 = 0;
         f.g3 = 0;
-        k_finalize_cols<<<ctx->t.Q * 3, kFinColThreads, 0, s>>>(ctx->b.part1, nullptr, nullptr, f, ctx->colsum, ctx->b.qcount + 3,
-                                                                ctx->series + ctx->T_out * ctx->rec_len);
+        // FP64 by k_finalize: where the nodes differ by rounding alone (FdPerNode) the record's variance over z
+        // shows the order of the sum
+        double *rec = ctx->series + ctx->T_out * ctx->rec_len;
+        if (ctx->cfg.precision == PGC_FP64)
+            k_finalize<<<1, kFinThreads, 0, s>>>(ctx->b.part1, nullptr, nullptr, f, rec);
+        else
+            k_finalize_cols<<<ctx->t.Q * 3, kFinColThreads, 0, s>>>(ctx->b.part1, nullptr, nullptr, f, ctx->colsum, ctx->b.qcount + 3, rec);
         count_launch();
         ctx->T_out++;
     }
