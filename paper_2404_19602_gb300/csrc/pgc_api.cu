@@ -864,9 +864,9 @@ pgc_status pgc_step(pgc_ctx *ctx, int64_t n_steps, int32_t moments_every)
     f.g1 = ctx->run->grid1();
     f.g2 = ctx->run->grid2();
     auto is_out = [&](int64_t n) { return moments_every > 0 && ((n + 1) % moments_every == 0); };
-    auto hist_max = [&](int64_t n) {
-        if (ctx->t.pauli_mode != PGC_PAULI_CURRENT_MAX) return;
-        launch_hist_max(ctx->b.hist + (int64_t)(n % kHistBufs) * ctx->b.hist_stride, ctx->t.Q, cells, ctx->b.nmax, s);
+    auto hist_max = [&](int64_t n) -> cudaError_t {
+        if (ctx->t.pauli_mode != PGC_PAULI_CURRENT_MAX) return cudaSuccess;
+        return launch_hist_max(ctx->b.hist + (int64_t)(n % kHistBufs) * ctx->b.hist_stride, ctx->t.Q, cells, ctx->b.nmax, s);
     };
     // record of step n: phase-1 partials of step n (g1 blocks), phase-2 partials of step n (g2
     // blocks) and, when phase 2 of step n - 1 carried particles into step n, its partials of step
@@ -929,7 +929,7 @@ pgc_status pgc_step(pgc_ctx *ctx, int64_t n_steps, int32_t moments_every)
     if (e == cudaSuccess && !pipelined) {
         for (int64_t k = 0; k < n_steps && e == cudaSuccess; ++k) {
             const int64_t n = n0 + k;
-            hist_max(n);
+            if ((e = hist_max(n)) != cudaSuccess) break;
             cudaEvent_t *ev = nullptr;
             if ((e = prof_slot(n, &ev)) != cudaSuccess) break;
             if ((e = before_writing(n)) != cudaSuccess) break;
@@ -944,12 +944,10 @@ pgc_status pgc_step(pgc_ctx *ctx, int64_t n_steps, int32_t moments_every)
         const int64_t n1 = n0 + n_steps - 1;
         // the bitmap of step n0 may hold bits left by steps taken outside this context's kernels
         e = cudaMemsetAsync(ctx->b.marks + (n0 % kMarkSlots) * ctx->b.mark_words, 0, (size_t)ctx->b.mark_words * 4, s);
-        if (e == cudaSuccess) {
-            hist_max(n0);
-            e = ctx->run->phase1(n0, is_out(n0), s);
-        }
+        if (e == cudaSuccess) e = hist_max(n0);
+        if (e == cudaSuccess) e = ctx->run->phase1(n0, is_out(n0), s);
         for (int64_t n = n0 + 1; n <= n1 && e == cudaSuccess; ++n) {
-            hist_max(n - 1);
+            if ((e = hist_max(n - 1)) != cudaSuccess) break;
             cudaEvent_t *ev = nullptr;
             if ((e = prof_slot(n, &ev)) != cudaSuccess) break;
             if ((e = before_writing(n)) != cudaSuccess) break;
@@ -959,8 +957,8 @@ pgc_status pgc_step(pgc_ctx *ctx, int64_t n_steps, int32_t moments_every)
             if (e == cudaSuccess && is_out(n - 1)) e = finalize_async(n - 1, g2f, n - 1 > n0 ? g2f : 0);
         }
         if (e == cudaSuccess) {
-            hist_max(n1);
-            e = before_writing(n1);
+            e = hist_max(n1);
+            if (e == cudaSuccess) e = before_writing(n1);
             if (e == cudaSuccess) e = ctx->run->phase2(n1, is_out(n1), s);
             if (e == cudaSuccess && is_out(n1)) e = finalize_async(n1, g2, n1 > n0 ? g2f : 0);
         }
