@@ -432,6 +432,32 @@ __device__ __forceinline__ void recon_all_rolled(const Nodes<P, Q, R> &nd, const
                 f(q1 * 6 + q2, kx, ky);
             }
         }
+    } else if constexpr (TensorShape<P, Q>::value) {
+#pragma unroll 1
+        for (int q1 = 0; q1 < 6; ++q1) {
+            R tx[6], ty[6];
+#pragma unroll
+            for (int h2 = 0; h2 < 6; ++h2) {
+                R sx = (R)0, sy = (R)0;
+#pragma unroll
+                for (int h1 = 0; h1 + h2 <= 5; ++h1) {
+                    sx += cx[hidx2(h1, h2)] * nd.a1[q1 * 6 + h1];
+                    sy += cy[hidx2(h1, h2)] * nd.a1[q1 * 6 + h1];
+                }
+                tx[h2] = sx;
+                ty[h2] = sy;
+            }
+#pragma unroll
+            for (int q2 = 0; q2 < 6; ++q2) {
+                R kx = (R)0, ky = (R)0;
+#pragma unroll
+                for (int h2 = 0; h2 < 6; ++h2) {
+                    kx += tx[h2] * nd.b2[q2 * 6 + h2];
+                    ky += ty[h2] * nd.b2[q2 * 6 + h2];
+                }
+                f(q1 * 6 + q2, kx, ky);
+            }
+        }
     } else {
 #pragma unroll 1
         for (int q = 0; q < Q; ++q) {
