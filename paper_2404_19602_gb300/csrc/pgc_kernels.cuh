@@ -365,22 +365,18 @@ __device__ __forceinline__ uint32_t window_code(float kx, float ky, unsigned lon
     const F2 s = f2_add_rd(f2_mul(f2_add(f2_pack(kx, ky), lk2), inv2), magic2);
     return (uint32_t)s.v * (4u * W) + (uint32_t)(s.v >> 32);
 }
-// The same for the FP64 mode from the node value rounded to FP32, with the distance of the FP32 cell
-// coordinates from the nearest cell edge (in `edge`, the smallest so far): the FP64 cell is the same
-// unless that distance is within the rounding (kCellGuard * Nk cells).
-constexpr float kCellGuard = 1e-6f;   // of Nk: four roundings of 6e-8 Nk, four times over
-template <int W>
-__device__ __forceinline__ uint32_t window_code_f64(double kx, double ky, unsigned long long lk2, F2 inv2, int win_r0, float &edge)
+// The FP64 mode's cell (row << 16 | column, 0xffffffff outside the grid) from the node value rounded to FP32; `near`
+// is set where the FP32 coordinates lie within their rounding of a cell edge (also for NaN and infinities):
+// elsewhere the FP64 cell is the same.
+constexpr float kCellGuard = 4e-7f;   // of Nk cells: four roundings of 2^-24 of at most Nk cells (2.4e-7) and as much again
+__device__ __forceinline__ uint32_t cell_code_f64(double kx, double ky, unsigned long long lk2, F2 inv2, int Nk, float guard, bool &near)
 {
-    const float m = 8388608.0f - (float)win_r0;
-    const F2 y = f2_mul(f2_add(f2_pack((float)kx, (float)ky), lk2), inv2);
-    const F2 s = f2_add_rd(y, f2_pack(m, m));
-    float yx, yy, sx, sy;
-    f2_unpack(y, yx, yy);
-    f2_unpack(s, sx, sy);
-    const float fx = yx - (float)win_r0 - (sx - 8388608.0f), fy = yy - (float)win_r0 - (sy - 8388608.0f);
-    edge = fminf(edge, fminf(fminf(fx, 1.0f - fx), fminf(fy, 1.0f - fy)));
-    return (uint32_t)s.v * (4u * W) + 4u * (uint32_t)(s.v >> 32);
+    float yx, yy;
+    f2_unpack(f2_mul(f2_add(f2_pack((float)kx, (float)ky), lk2), inv2), yx, yy);
+    const float fx = yx - floorf(yx), fy = yy - floorf(yy);
+    near = !(fminf(fminf(fx, 1.0f - fx), fminf(fy, 1.0f - fy)) > guard);
+    const int r = __float2int_rd(yx), l = __float2int_rd(yy);
+    return (unsigned)r < (unsigned)Nk && (unsigned)l < (unsigned)Nk ? ((uint32_t)r << 16) | (uint32_t)l : 0xffffffffu;
 }
 __device__ __forceinline__ F2 window_magic(int r0) { return f2_pack(8388608.0f - (float)r0, 2097152.0f - (float)r0); }
 
@@ -560,6 +556,35 @@ __device__ __forceinline__ void recon_at(const Nodes<P, Q, R> &nd, int q, const 
     }
 }
 
+// The same from a particle's stored coefficients (k: its column of [2P][ld]).
+template <int P, int Q, typename R>
+__device__ __forceinline__ void recon_stored(const Nodes<P, Q, R> &nd, int q, const R *k, int64_t ld, R &kx, R &ky)
+{
+    R sx2 = (R)0, sy2 = (R)0;
+    if constexpr (TensorShape<P, Q>::value) {
+        const int q1 = q / 6, q2 = q - 6 * (q / 6);
+#pragma unroll 1
+        for (int h2 = 0; h2 < 6; ++h2) {
+            R sx = (R)0, sy = (R)0;
+            for (int h1 = 0; h1 + h2 <= 5; ++h1) {
+                const int h = hidx2(h1, h2);
+                sx += k[(int64_t)h * ld] * nd.a1[q1 * 6 + h1];
+                sy += k[(int64_t)(P + h) * ld] * nd.a1[q1 * 6 + h1];
+            }
+            sx2 += sx * nd.b2[q2 * 6 + h2];
+            sy2 += sy * nd.b2[q2 * 6 + h2];
+        }
+    } else {
+#pragma unroll 4
+        for (int h = 0; h < P; ++h) {
+            sx2 += k[(int64_t)h * ld] * nd.psi[q * P + h];
+            sy2 += k[(int64_t)(P + h) * ld] * nd.psi[q * P + h];
+        }
+    }
+    kx = sx2;
+    ky = sy2;
+}
+
 // group velocity (units of vF) and energy at one node (Sec. 2).  The warp partial sums are
 // taken in R (FP32 in the production mode, FP64 in the FP64 mode) and accumulated in FP64.
 template <typename R>
@@ -693,33 +718,61 @@ __device__ __forceinline__ void queue_block(uint32_t *qcount, uint32_t *queue, c
     if (lane < n) queue[s_base[nw] + s_base[warp] + lane] = list[lane];
 }
 
-// Counts the histogram cells of n <= 32 such particles (one per lane) from their stored state.
+// Counts the cell of node q's value in the window or in the global histogram; 1 if it is outside the grid.
+template <int Q, int W, typename R>
+__device__ __forceinline__ unsigned int count_cell(const Phys<R> &ph, R lkx, int q, R kx, R ky, uint32_t *swin, int win_r0, bool use_win,
+                                                   uint32_t *Hnext)
+{
+    int r, l;
+    if (!cell_rl(ph, lkx, kx, ky, r, l)) return 1u;
+    const int rr = r - win_r0, ll = l - win_r0;
+    if (use_win && (unsigned)rr < (unsigned)W && (unsigned)ll < (unsigned)W)
+        atomicAdd(&swin[(q >> 1) * (W * W) + rr * W + ll], 1u << ((q & 1) << 4));
+    else
+        atomicAdd(&Hnext[((int64_t)q * ph.Nk + r) * ph.Nk + l], 1u);
+    return 0u;
+}
+
+// FP64: counts the nodes in `nodes` of one particle from its stored coefficients (k: its column).  Not inlined and
+// with no copy of the coefficients: it seldom runs, and the streaming pass has no registers for it.
+template <int P, int Q, int W>
+__device__ __noinline__ unsigned int count_nodes(const Phys<double> &ph, const Nodes<P, Q, double> &nd, const double *k, int64_t ld,
+                                                 uint64_t nodes, uint32_t *swin, int win_r0, bool use_win, uint32_t *Hnext)
+{
+    unsigned int oog = 0u;
+#pragma unroll 1
+    for (; nodes; nodes &= nodes - 1) {
+        const int q = __ffsll((long long)nodes) - 1;
+        double kx, ky;
+        recon_stored(nd, q, k, ld, kx, ky);
+        oog += count_cell<Q, W, double>(ph, nd.lkx[q], q, kx, ky, swin, win_r0, use_win, Hnext);
+    }
+    return oog;
+}
+
+// Counts the histogram cells of n <= 32 such particles (one per lane) from their stored state (FP32: the FP64
+// mode puts none aside).
 template <int P, int Q, typename R, int W>
 __device__ __forceinline__ void count_aside(const Phys<R> &ph, const Nodes<P, Q, R> &nd, const P1Target<R> &t, const uint32_t *list,
                                             int n, uint32_t *swin, int win_r0, bool use_win, unsigned int &oog)
 {
-    const int lane = threadIdx.x & 31;
-    const int64_t NN = (int64_t)ph.Nk * ph.Nk;
-    __syncwarp();   // the list and the drifted coefficients, written by other lanes
-    if (lane < n) {
-        const int64_t i = list[lane];
-        R cx[P], cy[P];
+    if constexpr (sizeof(R) == 4) {
+        const int lane = threadIdx.x & 31;
+        __syncwarp();   // the list and the drifted coefficients, written by other lanes
+        if (lane < n) {
+            const int64_t i = list[lane];
+            R cx[P], cy[P];
 #pragma unroll
-        for (int h = 0; h < P; ++h) {
-            cx[h] = t.khat[(int64_t)h * t.ld + i];
-            cy[h] = t.khat[(int64_t)(P + h) * t.ld + i];
+            for (int h = 0; h < P; ++h) {
+                cx[h] = t.khat[(int64_t)h * t.ld + i];
+                cy[h] = t.khat[(int64_t)(P + h) * t.ld + i];
+            }
+            recon_all_rolled(nd, cx, cy, [&](int q, R kx, R ky) {
+                oog += count_cell<Q, W, R>(ph, nd.lkx[q], q, kx, ky, swin, win_r0, use_win, t.Hnext);
+            });
         }
-        recon_all_rolled(nd, cx, cy, [&](int q, R kx, R ky) {
-            int r, l;
-            if (!cell_rl(ph, nd.lkx[q], kx, ky, r, l)) { ++oog; return; }
-            const int rr = r - win_r0, ll = l - win_r0;
-            if (use_win && (unsigned)rr < (unsigned)W && (unsigned)ll < (unsigned)W)
-                atomicAdd(&swin[(q >> 1) * (W * W) + rr * W + ll], 1u << ((q & 1) << 4));
-            else
-                atomicAdd(&t.Hnext[(int64_t)q * NN + r * ph.Nk + l], 1u);
-        });
+        __syncwarp();   // the list may be written again
     }
-    __syncwarp();   // the list may be written again
 }
 
 // One pass of a block over blockDim * PPT consecutive particles starting at i0 + threadIdx*PPT:
@@ -774,7 +827,7 @@ __device__ __forceinline__ void phase1_pass(const Phys<R> &ph, const Nodes<P, Q,
                 }
             }
     }
-    constexpr bool kUnrollQ = P * Q <= 64 || TensorShape<P, Q>::value;
+    constexpr bool kUnrollQ = P * Q <= 64 || (TensorShape<P, Q>::value && sizeof(R) == 4);
 #pragma unroll
     for (int e = 0; e < PPT; ++e) {
         const int64_t i = i0 + e;
@@ -783,6 +836,8 @@ __device__ __forceinline__ void phase1_pass(const Phys<R> &ph, const Nodes<P, Q,
         if (any && i < t.N && !((skipbits >> e) & 1u)) {
             // reconstruction, cells and the bound on the majorant
             uint32_t cell[Q];   // window_code
+            using NearMask = typename std::conditional<(Q > 32), uint64_t, uint32_t>::type;
+            NearMask near = 0;   // FP64: nodes whose cell FP32 does not decide
             const F2 inv2 = sizeof(R) == 4 ? f2_pack((float)ph.inv_dk, (float)ph.inv_dk) : f2_pack(ph.f.inv_dk, ph.f.inv_dk);
             const U4 r = philox4x32_10((uint32_t)i, t.stream_id, t.step, 0u, t.key0, t.key1);
             bool in_window;
@@ -813,14 +868,23 @@ __device__ __forceinline__ void phase1_pass(const Phys<R> &ph, const Nodes<P, Q,
                 maybe = screen_maybe(ph, nd, km.m, r.x);
             } else {
                 // FP64: cells and screen in FP32 where FP32 is certain of them (the FP64 pipe issues one warp
-                // instruction per 16 clocks; the reconstruction is what it has to do), else in FP64
+                // instruction per 16 clocks; the reconstruction is what it has to do), else in FP64: a node near a
+                // cell edge (one in 2500 at 240 cells) by itself.  No particle is formed a second time: the
+                // pipe is busy as long for one lane as for 32, and with the particles near an edge or outside
+                // the window's circle put aside every warp had such a lane (us a launch, put aside / here: 31 nodes,
+                // 1e4 particles 297 / 165; 36 nodes, 4e4 358 / 140; 6 nodes, 1e6 at 1000 cells, 1e5 79 / 48).
                 KkMax km;
-                float edge = 1.0f;
-                recon_all(ndb, cx[e], cy[e], [&](int q, R kx, R ky) {
-                    cell[q] = window_code_f64<W>(kx, ky, ndb.lk2[q], inv2, win_r0, edge);
+                const float guard = kCellGuard * (float)ph.Nk;
+                auto node = [&](int q, R kx, R ky) {
+                    bool nr;
+                    cell[q] = cell_code_f64(kx, ky, ndb.lk2[q], inv2, ph.Nk, guard, nr);
+                    near |= (NearMask)nr << q;
                     const float xf = (float)kx, yf = (float)ky;
                     km.add(q, Q, xf * xf + yf * yf);
-                });
+                };
+                // (36 nodes row by row: unrolled, the values of all nodes were held at once and 3 KB a thread spilled)
+                if constexpr (TensorShape<P, Q>::value) recon_all_rolled(ndb, cx[e], cy[e], node);
+                else recon_all(ndb, cx[e], cy[e], node);
                 const int sc = screen_f32(ph.f, km.n, (float)nd.eps0_max, r.x);
                 maybe = sc > 0;
                 if (sc < 0) {
@@ -828,21 +892,33 @@ __device__ __forceinline__ void phase1_pass(const Phys<R> &ph, const Nodes<P, Q,
                     recon_all_rolled(ndb, cx[e], cy[e], [&](int, R kx, R ky) { kk = fmax(kk, knorm2(kx, ky)); });
                     maybe = screen_maybe(ph, nd, kk, r.x);
                 }
-                in_window = km.n <= kk_in && edge > kCellGuard * (float)ph.Nk;
+                in_window = true;   // (each node is looked at below)
             }
             if (!maybe) {
                 finished[e] = true;
-                if (in_window) {   // every node value lies in the window
+                if (in_window) {
 #pragma unroll (kUnrollQ ? Q : 1)
-                    for (int q = 0; q < Q; ++q)
-                        atomicAdd(reinterpret_cast<uint32_t *>(reinterpret_cast<char *>(swin + (q >> 1) * (W * W)) + (cell[q] & 0xfffcu)),
-                                  (q & 1) ? 0x10000u : 1u);
+                    for (int q = 0; q < Q; ++q) {
+                        if constexpr (sizeof(R) == 4) {   // every node value lies in the window
+                            atomicAdd(reinterpret_cast<uint32_t *>(reinterpret_cast<char *>(swin + (q >> 1) * (W * W)) + (cell[q] & 0xfffcu)),
+                                      (q & 1) ? 0x10000u : 1u);
+                        } else if (!((near >> q) & 1)) {
+                            if (cell[q] == 0xffffffffu) { ++oog; continue; }
+                            const int r = (int)(cell[q] >> 16), l = (int)(cell[q] & 0xffffu), rr = r - win_r0, ll = l - win_r0;
+                            if (use_win && (unsigned)rr < (unsigned)W && (unsigned)ll < (unsigned)W)
+                                atomicAdd(&swin[(q >> 1) * (W * W) + rr * W + ll], 1u << ((q & 1) << 4));
+                            else
+                                atomicAdd(&t.Hnext[((int64_t)q * ph.Nk + r) * ph.Nk + l], 1u);
+                        }
+                    }
+                    if constexpr (sizeof(R) == 8)
+                        if (near) oog += count_nodes<P, Q, W>(ph, ndb, t.khat + i, t.ld, near, swin, win_r0, use_win, t.Hnext);
                 } else {
                     put_aside = true;
                 }
             }
         }
-        {
+        if (sizeof(R) == 4) {
             const unsigned int am = __ballot_sync(0xffffffffu, put_aside);
             if (am) {
                 if (put_aside) aside[n_aside + __popc(am & ((1u << lane) - 1u))] = (uint32_t)i;

@@ -1,6 +1,6 @@
 """The node values of a particle are formed at several places of the streaming kernels: unrolled
 (recon_all), rolled (recon_all_rolled: the particles counted again, the screen taken in FP64) and one
-node at a time (recon_at).  A cell or a screen may be decided by any of them, so they are the same
+node at a time (recon_at; recon_stored: the FP64 nodes near a cell edge).  A cell or a screen may be decided by any of them, so they are the same
 operations in the same order: bit for bit equal, for every kind of shape in both precisions, over
 ordinary coefficients and over ones of which the sums cancel.  The functions are compiled from the
 library's header into a program of their own."""
@@ -18,18 +18,21 @@ SRC = r"""
 using namespace pgc;
 
 template <int P, int Q, typename R>
-__global__ void k_three(const __grid_constant__ Nodes<P, Q, R> nd, const R *c, R *out, int n)
+__global__ void k_forms(const __grid_constant__ Nodes<P, Q, R> nd, const R *c, R *out, int n)
 {
     const int i = blockIdx.x * blockDim.x + threadIdx.x;
     if (i >= n) return;
     R cx[P], cy[P];
 #pragma unroll
     for (int h = 0; h < P; ++h) { cx[h] = c[(size_t)h * n + i]; cy[h] = c[(size_t)(P + h) * n + i]; }
-    R *o = out + (size_t)i * 6 * Q;
+    R *o = out + (size_t)i * 8 * Q;
     recon_all(nd, cx, cy, [&](int q, R kx, R ky) { o[q] = kx; o[Q + q] = ky; });
     recon_all_rolled(nd, cx, cy, [&](int q, R kx, R ky) { o[2 * Q + q] = kx; o[3 * Q + q] = ky; });
 #pragma unroll 1
-    for (int q = 0; q < Q; ++q) recon_at(nd, q, cx, cy, o[4 * Q + q], o[5 * Q + q]);
+    for (int q = 0; q < Q; ++q) {
+        recon_at(nd, q, cx, cy, o[4 * Q + q], o[5 * Q + q]);
+        if constexpr (sizeof(R) == 8) recon_stored(nd, q, c + i, (int64_t)n, o[6 * Q + q], o[7 * Q + q]);
+    }
 }
 
 template <int P, int Q, typename R>
@@ -56,20 +59,21 @@ static long differ(int n, double spread)
         for (int j = 0; j < Q * P; ++j) nd.psi2[j] = pair((float)nd.psi[j]);
     std::vector<R> c((size_t)2 * P * n);
     for (R &v : c) v = (R)(z(g) * std::pow(10.0, spread * z(g)));
-    std::vector<R> out((size_t)6 * Q * n);
+    std::vector<R> out((size_t)8 * Q * n);
     R *dc = nullptr, *dout = nullptr;
     if (cudaMalloc(&dc, c.size() * sizeof(R)) || cudaMalloc(&dout, out.size() * sizeof(R)) ||
         cudaMemcpy(dc, c.data(), c.size() * sizeof(R), cudaMemcpyHostToDevice)) return -1;
-    k_three<P, Q, R><<<(n + 127) / 128, 128>>>(nd, dc, dout, n);
+    k_forms<P, Q, R><<<(n + 127) / 128, 128>>>(nd, dc, dout, n);
     if (cudaGetLastError() || cudaMemcpy(out.data(), dout, out.size() * sizeof(R), cudaMemcpyDeviceToHost)) return -1;
     cudaFree(dc);
     cudaFree(dout);
     long bad = 0;
     for (int i = 0; i < n; ++i)
         for (int j = 0; j < 2 * Q; ++j) {
-            const R *o = &out[(size_t)i * 6 * Q];
+            const R *o = &out[(size_t)i * 8 * Q];
             bad += !(o[j] == o[2 * Q + j]);
             bad += !(o[j] == o[4 * Q + j]);
+            if (sizeof(R) == 8) bad += !(o[j] == o[6 * Q + j]);
         }
     return bad;
 }

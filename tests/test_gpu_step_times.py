@@ -1,0 +1,60 @@
+"""Times of a step that must not depend on what they once depended on, as ratios of two runs in one
+process (medians of event-timed steps; the bounds leave a margin of a fifth or more over what is
+expected, and a quarter or more below what the former kernels took)."""
+import numpy as np
+import pytest
+
+from paper_2404_19602_gb300 import workloads as W
+
+pytestmark = pytest.mark.gpu
+torch = pytest.importorskip("torch")
+
+
+def _step_us(sim, steps=20, runs=15):
+    sim.step(steps, 0)
+    got = []
+    for _ in range(runs):
+        a, b = torch.cuda.Event(enable_timing=True), torch.cuda.Event(enable_timing=True)
+        a.record()
+        sim.step(steps, 0)
+        b.record()
+        b.synchronize()
+        got.append(a.elapsed_time(b) * 1e3 / steps)
+    return sorted(got)[runs // 2]
+
+
+@pytest.fixture(scope="module", autouse=True)
+def _built():
+    from paper_2404_19602_gb300 import build
+
+    if not torch.cuda.is_available():
+        pytest.skip("no CUDA device")
+    build.build()
+
+
+@pytest.mark.parametrize("shape", ["31x31", "21x36"])
+def test_fp64_cell_edges_and_far_states_cost_little(shape):
+    """FP64: an ensemble spread over the grid, some values next to cell edges and some outside the
+    shared-memory window, against the same ensemble at cell centres near the middle.  Counted a second
+    time as whole particles these cost 1.5 to 1.9 times a launch."""
+    from paper_2404_19602_gb300 import pgc
+
+    kw = dict(N=1000, precision="fp64", seed=3, mech_mask=0, Ex_lo=0.0)
+    p = W.scaled(W.TEST2_WIDTH_1E6, M=30, Q1=31, Ex_hi=0.0, **kw) if shape == "31x31" else W.scaled(W.GAP_FIELD_UQ_4E6, Ex_hi=1e-9, **kw)
+    Lk = p["Lk_hvF"] / (6.582119569e-16 * 1e6 * 1e9)
+    dk = 2 * Lk / p["Nk"]
+    rng = np.random.default_rng(1)
+    us = []
+    for spread in (0, 1):
+        sim = pgc.Simulation(p, max_outputs=4)
+        k = np.zeros((2, sim.P, p["N"]))
+        k[:, 0] = (rng.integers(-8, 8, (2, p["N"])) + 0.5) * dk
+        if spread:
+            k[:, 0] = rng.uniform(-14, 14, (2, p["N"])) * dk
+            k[:, 0, ::20] *= 2.5
+            k[0, 1] = 1e-3 * rng.standard_normal(p["N"])
+        sim.set_state(k)
+        us.append(_step_us(sim))
+        sim.close()
+    print(shape, us)
+    assert us[1] <= 1.25 * us[0]
