@@ -345,12 +345,12 @@ public:
         a_.done = sc.done;
         a_.moments_every = 0;
         constexpr int W = HistWin<P, Q, R>::batchW;
-        a_.use_win = t0.Nk >= W;
+        a_.use_win = 1;
         a_.win_r0 = window_r0(t0.Nk, W);
-        a_.kk_in = a_.use_win ? (float)window_kk(t0, W) : -1.0f;
+        a_.kk_in = (float)window_kk(t0, W);
         a_.rec_len = 1 + 4 * Q + 8;
         a_.vF_ms = t0.vF_ms;
-        win_bytes_ = a_.use_win ? HistWin<P, Q, R>::batch_bytes : 0;
+        win_bytes_ = HistWin<P, Q, R>::batch_bytes;
         num_sms_ = num_sms;
         for (int j = 0; j < BatchPPTs<P>::n; ++j)
             if (win_bytes_) cudaFuncSetAttribute(kernel1(BatchPPTs<P>::v[j]), cudaFuncAttributeMaxDynamicSharedMemorySize, (int)win_bytes_);
