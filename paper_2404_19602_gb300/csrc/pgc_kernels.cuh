@@ -43,11 +43,11 @@ constexpr int kGrid2Max = 5 * 152; // phase-2 partial sums are sized for this ma
 //   36 nodes, FP32: one block of 512 threads per SM owns one window of 48 x 48 cells (166 KB).  Two
 //   blocks with 32 x 32 each (+-0.67 eV) left 2-4 % of the particles with a node outside (3/4 of
 //   the warps had such a lane) once the field had heated the ensemble; 48 x 48 (+-1 eV): 0.1 %.
-//   One-dimensional shapes: 48 x 48 up to 6 nodes (28 KB), else 40 x 40 (31 nodes 102 KB); 36 nodes
-//   FP64: 32 x 32.
+//   One-dimensional shapes: 48 x 48 up to 6 nodes (28 KB), 40 x 40 up to 26 (83 KB), 36 x 36 at 31 (83 KB: two
+//   blocks per SM; 40 x 40, 102 KB, left one in FP32); 36 nodes FP64: 32 x 32.
 template <int P, int Q, typename R> struct HistWin {
     static constexpr int pairs = (Q + 1) / 2;
-    static constexpr int W = (Q == 36) ? (sizeof(R) == 4 ? 48 : 32) : (Q <= 6 ? 48 : 40);
+    static constexpr int W = (Q == 36) ? (sizeof(R) == 4 ? 48 : 32) : (Q <= 6 ? 48 : Q <= 26 ? 40 : 36);
     static constexpr size_t bytes = (size_t)pairs * W * W * 4;
     // the batched kernel (blocks of up to 256 threads, two per SM at 36 nodes)
     static constexpr int batchW = (Q == 36) ? (sizeof(R) == 4 ? 36 : 32) : 56;
@@ -614,10 +614,12 @@ __device__ __forceinline__ void observe_fast(const Phys<float> &ph, float kx, fl
 // ------------------------------------------------------------------------------------------
 template <int P> struct Phase1PPT { static constexpr int value = (P <= 8) ? 4 : 1; };
 // resident blocks per SM the streaming kernels are compiled for: three for the small FP32
-// shapes, two (more registers, no spills) for the large shapes and for FP64; one block of 512
-// threads for 36 nodes in FP32 (the same 128 registers, one window per SM)
+// shapes, two (more registers, fewer spills) for the large shapes and for FP64; one block of 512
+// threads for 36 nodes in FP32 (the same 128 registers, one window per SM).  k_phase1 alone also three at 9
+// nodes (it fits; 1e6 particles 59 us a launch with two, 55 with three).
 template <int P, int Q, typename R> struct kPhase1MinBlocks {
     static constexpr int value = (Q == 36 && sizeof(R) == 4) ? 1 : (P * Q > 64 || sizeof(R) == 8) ? 2 : 3;
+    static constexpr int phase1 = (sizeof(R) == 4 && P * Q <= 100) ? 3 : value;
 };
 
 template <typename R, int PPT>
@@ -686,7 +688,12 @@ struct P1Target {
 
 // The particles of a warp with a node value outside the circle of the window (kk_in), put aside in
 // shared memory: a rolled pass over their nodes for one lane costs a warp as much as for 32, so they
-// are taken 32 at a time (at most 31 stay between passes).
+// are taken 32 at a time (at most 31 stay between passes).  Not in FP64 and not at the large one-dimensional
+// shapes: there the cells are a small part of a pass, and even the last incomplete list of a warp costs as much
+// as the pass itself, so each node's cell is checked against the window by itself (FP32, us a launch with
+// lists and one window per SM at 31 nodes / by node: 31 nodes 2e4 particles 33.5 / 23.6, 2e5 139 / 66;
+// 21 nodes 1e6 174 / 140).
+template <int P, int Q, typename R> struct PutsAside { static constexpr bool value = sizeof(R) == 4 && !StagePsi<P, Q, R>::value; };
 template <int PPT> struct AsideList { static constexpr int cap = 32 * (PPT + 1); };
 
 // The colliders a warp finds wait in a list of their own (also AsideList::cap entries) and reach the
@@ -750,13 +757,12 @@ __device__ __noinline__ unsigned int count_nodes(const Phys<double> &ph, const N
     return oog;
 }
 
-// Counts the histogram cells of n <= 32 such particles (one per lane) from their stored state (FP32: the FP64
-// mode puts none aside).
+// Counts the histogram cells of n <= 32 such particles (one per lane) from their stored state.
 template <int P, int Q, typename R, int W>
 __device__ __forceinline__ void count_aside(const Phys<R> &ph, const Nodes<P, Q, R> &nd, const P1Target<R> &t, const uint32_t *list,
                                             int n, uint32_t *swin, int win_r0, bool use_win, unsigned int &oog)
 {
-    if constexpr (sizeof(R) == 4) {
+    if constexpr (PutsAside<P, Q, R>::value) {
         const int lane = threadIdx.x & 31;
         __syncwarp();   // the list and the drifted coefficients, written by other lanes
         if (lane < n) {
@@ -828,6 +834,7 @@ __device__ __forceinline__ void phase1_pass(const Phys<R> &ph, const Nodes<P, Q,
             }
     }
     constexpr bool kUnrollQ = P * Q <= 64 || (TensorShape<P, Q>::value && sizeof(R) == 4);
+    constexpr bool kCells = !PutsAside<P, Q, R>::value;
 #pragma unroll
     for (int e = 0; e < PPT; ++e) {
         const int64_t i = i0 + e;
@@ -835,7 +842,7 @@ __device__ __forceinline__ void phase1_pass(const Phys<R> &ph, const Nodes<P, Q,
         bool maybe = false, put_aside = false;
         if (any && i < t.N && !((skipbits >> e) & 1u)) {
             // reconstruction, cells and the bound on the majorant
-            uint32_t cell[Q];   // window_code
+            uint32_t cell[Q];   // window_code, or with kCells row << 16 | column (0xffffffff outside the grid)
             using NearMask = typename std::conditional<(Q > 32), uint64_t, uint32_t>::type;
             NearMask near = 0;   // FP64: nodes whose cell FP32 does not decide
             const F2 inv2 = sizeof(R) == 4 ? f2_pack((float)ph.inv_dk, (float)ph.inv_dk) : f2_pack(ph.f.inv_dk, ph.f.inv_dk);
@@ -853,10 +860,9 @@ __device__ __forceinline__ void phase1_pass(const Phys<R> &ph, const Nodes<P, Q,
                         for (int h = 0; h < P; ++h) s2 = f2_fma(f2_pack(cx[e][h], cy[e][h]), (h & 1) ? w[h >> 1].y : w[h >> 1].x, s2);
                         float kx, ky;
                         f2_unpack(s2, kx, ky);
-                        cell[q] = window_code<W>(kx, ky, ndb.lk2[q], inv2, magic2);
-                        const float kk = knorm2(kx, ky);
-                        km.m = fmaxf(km.m, kk);
-                        km.n = max3_nan(km.n, kk, kk);
+                        int rw, cl;
+                        cell[q] = cell_rl(ph, ndb.lkx[q], kx, ky, rw, cl) ? ((uint32_t)rw << 16) | (uint32_t)cl : 0xffffffffu;
+                        km.m = fmaxf(km.m, knorm2(kx, ky));
                     }
                 } else {
                     recon_all(ndb, cx[e], cy[e], [&](int q, R kx, R ky) {
@@ -864,7 +870,7 @@ __device__ __forceinline__ void phase1_pass(const Phys<R> &ph, const Nodes<P, Q,
                         km.add(q, Q, knorm2(kx, ky));
                     });
                 }
-                in_window = km.n <= kk_in;   // (false for NaN)
+                in_window = kCells || km.n <= kk_in;   // (false for NaN)
                 maybe = screen_maybe(ph, nd, km.m, r.x);
             } else {
                 // FP64: cells and screen in FP32 where FP32 is certain of them (the FP64 pipe issues one warp
@@ -892,17 +898,17 @@ __device__ __forceinline__ void phase1_pass(const Phys<R> &ph, const Nodes<P, Q,
                     recon_all_rolled(ndb, cx[e], cy[e], [&](int, R kx, R ky) { kk = fmax(kk, knorm2(kx, ky)); });
                     maybe = screen_maybe(ph, nd, kk, r.x);
                 }
-                in_window = true;   // (each node is looked at below)
+                in_window = true;
             }
             if (!maybe) {
                 finished[e] = true;
                 if (in_window) {
 #pragma unroll (kUnrollQ ? Q : 1)
                     for (int q = 0; q < Q; ++q) {
-                        if constexpr (sizeof(R) == 4) {   // every node value lies in the window
+                        if constexpr (!kCells) {   // every node value lies in the window
                             atomicAdd(reinterpret_cast<uint32_t *>(reinterpret_cast<char *>(swin + (q >> 1) * (W * W)) + (cell[q] & 0xfffcu)),
                                       (q & 1) ? 0x10000u : 1u);
-                        } else if (!((near >> q) & 1)) {
+                        } else if (sizeof(R) == 4 || !((near >> q) & 1)) {
                             if (cell[q] == 0xffffffffu) { ++oog; continue; }
                             const int r = (int)(cell[q] >> 16), l = (int)(cell[q] & 0xffffu), rr = r - win_r0, ll = l - win_r0;
                             if (use_win && (unsigned)rr < (unsigned)W && (unsigned)ll < (unsigned)W)
@@ -918,7 +924,7 @@ __device__ __forceinline__ void phase1_pass(const Phys<R> &ph, const Nodes<P, Q,
                 }
             }
         }
-        if (sizeof(R) == 4) {
+        if (!kCells) {
             const unsigned int am = __ballot_sync(0xffffffffu, put_aside);
             if (am) {
                 if (put_aside) aside[n_aside + __popc(am & ((1u << lane) - 1u))] = (uint32_t)i;
@@ -1190,7 +1196,7 @@ __device__ __forceinline__ void phase1_block(const StepArgs<P, Q, R> &a, int bid
 }
 
 template <int P, int Q, typename R>
-__global__ void __launch_bounds__(P1Threads<P, Q, R>::value, kPhase1MinBlocks<P, Q, R>::value)
+__global__ void __launch_bounds__(P1Threads<P, Q, R>::value, kPhase1MinBlocks<P, Q, R>::phase1)
 k_phase1(const __grid_constant__ StepArgs<P, Q, R> a)
 {
     extern __shared__ __align__(16) uint32_t swin[];   // HistWin when a.use_win

@@ -58,3 +58,17 @@ def test_fp64_cell_edges_and_far_states_cost_little(shape):
         sim.close()
     print(shape, us)
     assert us[1] <= 1.25 * us[0]
+
+
+def test_fp32_31_nodes_against_26():
+    """FP32 streaming (no scattering) at 31 nodes against 26: the multiply-adds grow 1.42 times (31^2 / 26^2); with
+    one window per SM instead of two and a last incomplete list per warp it was over twice."""
+    from paper_2404_19602_gb300 import pgc
+
+    us = []
+    for M in (25, 30):
+        sim = pgc.Simulation(W.scaled(W.TEST2_WIDTH_1E6, N=200_000, M=M, Q1=M + 1, mech_mask=0, seed=3), max_outputs=4)
+        us.append(_step_us(sim))
+        sim.close()
+    print(us)
+    assert us[1] <= 1.75 * us[0]
