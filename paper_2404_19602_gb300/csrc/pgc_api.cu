@@ -712,7 +712,7 @@ static pgc_status observe_current(pgc_ctx *ctx, bool record, bool set_nmax)
         f.vF_ms = ctx->t.vF_ms;
         f.t_fs = ctx->step * ctx->t.dt;
         f.Q = ctx->t.Q;
-        f.g1 = ctx->run->grid1();
+        f.g1 = ctx->run->grid_obs();
         f.g2 = 0;
         f.g3 = 0;
         // FP64 by k_finalize: where the nodes differ by rounding alone (FdPerNode) the record's variance over z

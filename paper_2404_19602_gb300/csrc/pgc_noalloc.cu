@@ -54,7 +54,7 @@ extern "C" pgc_status pgc_observe_static(pgc_ctx *ctx, uint32_t *d_hist_out, dou
     if (!ctx) return PGC_EINVAL;
     if (ctx->failed) { ctx->err = "context failed earlier: " + ctx->err; return PGC_ESTATE; }
     if (!d_hist_out || !d_record_out) { ctx->err = "pgc_observe_static: output pointers must be non-NULL"; return PGC_EINVAL; }
-    const int Q = ctx->t.Q, g1 = ctx->run->grid1();
+    const int Q = ctx->t.Q, g1 = ctx->run->grid_obs();
     const size_t need = (size_t)g1 * Q * 3 * sizeof(double);
     if (need > kNoAllocBytes) {
         ctx->err = "pgc_observe_static: " + std::to_string(g1) + " blocks x " + std::to_string(Q) +

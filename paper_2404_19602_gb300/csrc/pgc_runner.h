@@ -68,6 +68,7 @@ class Runner {
 public:
     virtual ~Runner() {}
     virtual int grid1() const = 0;
+    virtual int grid_obs() const = 0;   // blocks of k_observe (rows of its partial sums)
     virtual int grid2() const = 0;
     virtual int grid2f() const = 0;   // phase-2 blocks of the fused step kernel
     // sample the Fermi-Dirac initial state into the state buffer
@@ -75,7 +76,7 @@ public:
     // histogram of the current state into hist buffer `buf` and moment partials into part1
     virtual cudaError_t observe(int buf, cudaStream_t s) = 0;
     // histogram of the current state into `hist` ([Q][Nk*Nk], zeroed by the caller) and moment
-    // partials into `part` ([grid1()][Q*3]); touches no context buffer
+    // partials into `part` ([grid_obs()][Q*3]); touches no context buffer
     virtual cudaError_t observe_into(uint32_t *hist, double *part, cudaStream_t s) = 0;
     // time step number `step` as two launches on one stream; if ev is non-NULL, ev[0..3] are
     // recorded before phase 1, after it, before phase 2 and after it

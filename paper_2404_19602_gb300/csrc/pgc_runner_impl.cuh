@@ -117,7 +117,13 @@ public:
         cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, k_phase1<P, Q, R>, T1, win ? win_bytes_ : 0);
         per_sm = std::max(per_sm, 1);
         const int64_t need = (b.N + (int64_t)T1 * PPT - 1) / ((int64_t)T1 * PPT);
-        grid1_ = (int)std::max<int64_t>(1, std::min<int64_t>({need, (int64_t)num_sms * per_sm, (int64_t)kMaxGrid1}));
+        const int64_t most = std::min<int64_t>((int64_t)num_sms * per_sm, kMaxGrid1);
+        grid_obs_ = (int)std::max<int64_t>(1, std::min(need, most));
+        // A step also clears f^{n+2}, whose size does not depend on N (36 nodes 8.3 MB, 6 nodes 1.4 MB): blocks
+        // beyond those that have particles take their share of it, so that none clears more than kClearBytes.  36
+        // nodes, 1e3 particles (2 blocks of 512 threads): 76 us a launch by those alone, 14 so; 31 nodes FP32 55, 21.
+        const int64_t clear = (args_.hist_elems * 4 + kClearBytes - 1) / kClearBytes;
+        grid1_ = (int)std::max<int64_t>(1, std::min(std::max(need, clear), most));
         args_.use_win = win ? 1 : 0;
         if (!win) win_bytes_ = 0;
         args_.kk_in = win ? (float)window_kk(t, W) : -1.0f;
@@ -130,6 +136,7 @@ public:
     }
 
     int grid1() const override { return grid1_; }
+    int grid_obs() const override { return grid_obs_; }
     int grid2() const override { return grid2_; }
     int grid2f() const override { return grid2f_; }
     const StepArgs<P, Q, R> &args() const { return args_; }
@@ -234,6 +241,7 @@ public:
             if (per_sm != 1) return cudaErrorNotSupported;   // TMEM is sized for one CTA per SM
             const int64_t tiles = (b_.N + 127) / 128;
             grid1_ = (int)std::max<int64_t>(1, std::min<int64_t>((tiles + kTcWG - 1) / kTcWG, num_sms_));
+            grid_obs_ = grid1_;
             args_.win_r0 = window_r0(t_.Nk, kWin);
             args_.use_win = t_.Nk >= kWin;
             tc_mode_ = mode;
@@ -379,7 +387,7 @@ private:
     void launch_observe(StepArgs<P, Q, R> &a, cudaStream_t s)
     {
         if (tc_mode_) a.use_win = 0;
-        k_observe<P, Q, R><<<grid1_, P1Threads<P, Q, R>::value, a.use_win ? win_bytes_ : 0, s>>>(a);
+        k_observe<P, Q, R><<<grid_obs_, P1Threads<P, Q, R>::value, a.use_win ? win_bytes_ : 0, s>>>(a);
     }
 
     void fill_phys(const HostTables &t)
@@ -441,7 +449,7 @@ private:
     StepArgs<P, Q, R> args_{};
     InitArgs<P, Q> init_{};
     std::vector<double> edge_host_;
-    int grid1_ = 1;
+    int grid1_ = 1, grid_obs_ = 1;
     size_t win_bytes_ = 0;
     int grid2_ = 1;
     int grid2f_ = 1;
