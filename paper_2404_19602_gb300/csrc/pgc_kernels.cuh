@@ -1101,15 +1101,12 @@ __device__ __forceinline__ void phase1_block(const StepArgs<P, Q, R> &a, int bid
     using SP = StagePsi<P, Q, R>;
     __shared__ __align__(16) unsigned long long spsi[SP::elems];
     const int64_t tile = (int64_t)blockDim.x * PPT;
-    const bool streams = a.tilectr || (int64_t)bid * tile < a.N;   // (else the block only clears)
-    const bool use_win = a.use_win && streams;
     if constexpr (SP::value)
-        if (streams)
+        if (a.tilectr || (int64_t)bid * tile < a.N)   // (a block without particles only clears)
             for (int j = threadIdx.x; j < Q * P; j += blockDim.x) {
                 const float w = a.nd_dev ? a.nd_dev->psi[j] : a.nd.psi[j];
                 spsi[(j / P) * SP::row + j % P] = f2_pack(w, w).v;
             }
-    if (use_win) clear_window<Q, HistWin<P, Q, R>::W>(swin);
     if (a.out_step)
         for (int j = lane; j < Q * 3; j += 32) acc_zero(smom[warp][j]);
     __syncthreads();
@@ -1140,13 +1137,16 @@ __device__ __forceinline__ void phase1_block(const StepArgs<P, Q, R> &a, int bid
     unsigned int oog = 0u;
     // A window cell holds 16 bits and a particle adds at most one count to a cell per node, so the
     // window is flushed to f^{n+1} before the block has counted 65535 particles since the last
-    // flush (block-uniform; with the tile counter a block may take any number of tiles).
+    // flush (block-uniform; with the tile counter a block may take any number of tiles).  A block
+    // without a tile has no window: it neither clears nor flushes one.
     int64_t since_flush = 0;
     auto guard_window = [&]() {
-        if (use_win && since_flush + tile + blockDim.x > 65535) {   // (blockDim.x: particles put aside before the flush)
-            __syncthreads();
-            flush_window<Q, HistWin<P, Q, R>::W>(swin, a.Hnext, a.ph.Nk, a.win_r0);
-            __syncthreads();
+        if (a.use_win && (since_flush == 0 || since_flush + tile + blockDim.x > 65535)) {   // (blockDim.x: particles put aside before the flush)
+            if (since_flush > 0) {
+                __syncthreads();
+                flush_window<Q, HistWin<P, Q, R>::W>(swin, a.Hnext, a.ph.Nk, a.win_r0);
+                __syncthreads();
+            }
             clear_window<Q, HistWin<P, Q, R>::W>(swin);
             __syncthreads();
             since_flush = 0;
@@ -1159,10 +1159,10 @@ __device__ __forceinline__ void phase1_block(const StepArgs<P, Q, R> &a, int bid
     auto pass = [&](int64_t base) {
         constexpr int W = HistWin<P, Q, R>::W;
         if (PPT == 1 || P > 1 || sizeof(R) == 8 || a.out_step) {
-            phase1_pass<P, Q, R, W, PPT>(a.ph, a.nd, a.nd, t, base + (int64_t)threadIdx.x * PPT, swin, a.win_r0, use_win, a.kk_in,
+            phase1_pass<P, Q, R, W, PPT>(a.ph, a.nd, a.nd, t, base + (int64_t)threadIdx.x * PPT, swin, a.win_r0, a.use_win != 0, a.kk_in,
                                          a.out_step != 0, smom[warp], aside, n_aside, qlist, n_q, oog, spsi);
         } else {
-            phase1_rolled<P, Q, R, W, PPT>(a.ph, a.nd, a.nd, t, base, swin, a.win_r0, use_win, a.kk_in, smom[warp], aside, n_aside,
+            phase1_rolled<P, Q, R, W, PPT>(a.ph, a.nd, a.nd, t, base, swin, a.win_r0, a.use_win != 0, a.kk_in, smom[warp], aside, n_aside,
                                            qlist, n_q, oog);
         }
     };
@@ -1184,11 +1184,11 @@ __device__ __forceinline__ void phase1_block(const StepArgs<P, Q, R> &a, int bid
         }
     }
     if (n_aside > 0)
-        count_aside<P, Q, R, HistWin<P, Q, R>::W>(a.ph, a.nd, t, aside, n_aside, swin, a.win_r0, use_win, oog);
+        count_aside<P, Q, R, HistWin<P, Q, R>::W>(a.ph, a.nd, t, aside, n_aside, swin, a.win_r0, a.use_win != 0, oog);
     oog = warp_sum(oog);
     if (lane == 0 && oog) atomicAdd(&a.counters[4], (unsigned long long)oog);
     queue_block(t.qcount, t.queue, qlist, n_q, s_qbase);   // (synchronises)
-    if (use_win) flush_window<Q, HistWin<P, Q, R>::W>(swin, a.Hnext, a.ph.Nk, a.win_r0);
+    if (a.use_win && since_flush > 0) flush_window<Q, HistWin<P, Q, R>::W>(swin, a.Hnext, a.ph.Nk, a.win_r0);
     if (a.out_step) {
         for (int j = threadIdx.x; j < Q * 3; j += blockDim.x) {
             double s = 0.0;
