@@ -1039,31 +1039,57 @@ __device__ __forceinline__ void phase1_rolled(const Phys<R> &ph, const Nodes<P, 
     }
 }
 
-// Clear a block's window; add it to the global histogram, one add per non-empty cell and node (the
-// words of the window are mostly empty: four are looked at per load).
+// Clear a block's window (dynamic shared memory).
 template <int Q, int W>
 __device__ __forceinline__ void clear_window(uint32_t *swin)
 {
+    static_assert(W % 4 == 0, "four cells of a row per access");
     for (int j = threadIdx.x; j < (Q + 1) / 2 * (W * W / 4); j += blockDim.x)
         reinterpret_cast<uint4 *>(swin)[j] = make_uint4(0u, 0u, 0u, 0u);
 }
 
+// Add it to the global histogram, one add per non-empty cell and node.  A lane takes one word, so that a warp's adds
+// fall on 32 cells side by side, four sectors of L2: with four cells a lane they fell on sixteen, and the
+// fuller the window the more the flush was the step (1e6 particles x 6 nodes, us a step: 240 cells 33.6 -> 32.2, after
+// 3000 steps 38.5 -> 35.9; 480 cells 48.2 -> 36.4; 600 cells 57 -> 41).  A sparse window at 36 nodes (the
+// block has counted fewer than kSparseWindow particles) is looked at four words a load all the same, since there the
+// words looked at are the cost (2e5 particles, 1300 a block: 27.5 us a launch, 29.0 word by word; at 4e6 the
+// two are equal).  Not inlined: the streaming loop has no register to spare for it.
+constexpr int kSparseWindow = 2000;
 template <int Q, int W>
-__device__ __forceinline__ void flush_window(const uint32_t *swin, uint32_t *Hnext, int Nk, int win_r0)
+__device__ __noinline__ void flush_window(uint32_t *Hnext, int Nk, int win_r0, int64_t counted)
 {
-    static_assert(W % 4 == 0, "four cells of a row per load");
-    const int64_t NN = (int64_t)Nk * Nk;
-    for (int j = threadIdx.x; j < (Q + 1) / 2 * (W * W / 4); j += blockDim.x) {
-        const uint4 v4 = reinterpret_cast<const uint4 *>(swin)[j];
-        if (!(v4.x | v4.y | v4.z | v4.w)) continue;
-        const int p = j / (W * W / 4), w = j % (W * W / 4);
-        uint32_t *base = Hnext + (int64_t)(2 * p) * NN + (int64_t)(w / (W / 4) + win_r0) * Nk + 4 * (w % (W / 4)) + win_r0;
-        const uint32_t v[4] = {v4.x, v4.y, v4.z, v4.w};
-#pragma unroll
-        for (int c = 0; c < 4; ++c) {
-            if (v[c] & 0xffffu) atomicAdd(base + c, v[c] & 0xffffu);
-            if (v[c] >> 16) atomicAdd(base + NN + c, v[c] >> 16);
+    extern __shared__ __align__(16) uint32_t swin[];
+    constexpr uint32_t n = (Q + 1) / 2 * W * W, U = Q > 6 ? 8 : 4;
+    const uint32_t NN = (uint32_t)Nk * Nk, pair = 2 * NN - W * (uint32_t)Nk;   // (a histogram of all nodes has < 2^32 cells)
+    uint32_t *base = Hnext + win_r0 * (Nk + 1);
+    auto cell = [&](uint32_t j) {
+        const uint32_t r = j / W, p = r / W;   // row of all pairs' windows, node pair
+        return base + (size_t)(p * pair + r * (uint32_t)Nk + (j - r * W));
+    };
+    auto add = [&](uint32_t *h, uint32_t v) {
+        if (v & 0xffffu) atomicAdd(h, v & 0xffffu);
+        if (v >> 16) atomicAdd(h + NN, v >> 16);
+    };
+    if (Q == 36 && counted < kSparseWindow) {
+        for (uint32_t j = threadIdx.x; j < n / 4; j += blockDim.x) {
+            const uint4 v = reinterpret_cast<const uint4 *>(swin)[j];
+            if (!(v.x | v.y | v.z | v.w)) continue;
+            uint32_t *h = cell(4 * j);
+            add(h, v.x);
+            add(h + 1, v.y);
+            add(h + 2, v.z);
+            add(h + 3, v.w);
         }
+        return;
+    }
+    for (uint32_t j0 = threadIdx.x; j0 < n; j0 += U * blockDim.x) {
+        uint32_t v[U];
+#pragma unroll
+        for (uint32_t u = 0; u < U; ++u) v[u] = j0 + u * blockDim.x < n ? swin[j0 + u * blockDim.x] : 0u;
+#pragma unroll
+        for (uint32_t u = 0; u < U; ++u)
+            if (v[u]) add(cell(j0 + u * blockDim.x), v[u]);
     }
 }
 
@@ -1144,7 +1170,7 @@ __device__ __forceinline__ void phase1_block(const StepArgs<P, Q, R> &a, int bid
         if (a.use_win && (since_flush == 0 || since_flush + tile + blockDim.x > 65535)) {   // (blockDim.x: particles put aside before the flush)
             if (since_flush > 0) {
                 __syncthreads();
-                flush_window<Q, HistWin<P, Q, R>::W>(swin, a.Hnext, a.ph.Nk, a.win_r0);
+                flush_window<Q, HistWin<P, Q, R>::W>(a.Hnext, a.ph.Nk, a.win_r0, since_flush);
                 __syncthreads();
             }
             clear_window<Q, HistWin<P, Q, R>::W>(swin);
@@ -1188,7 +1214,7 @@ __device__ __forceinline__ void phase1_block(const StepArgs<P, Q, R> &a, int bid
     oog = warp_sum(oog);
     if (lane == 0 && oog) atomicAdd(&a.counters[4], (unsigned long long)oog);
     queue_block(t.qcount, t.queue, qlist, n_q, s_qbase);   // (synchronises)
-    if (a.use_win && since_flush > 0) flush_window<Q, HistWin<P, Q, R>::W>(swin, a.Hnext, a.ph.Nk, a.win_r0);
+    if (a.use_win && since_flush > 0) flush_window<Q, HistWin<P, Q, R>::W>(a.Hnext, a.ph.Nk, a.win_r0, since_flush);
     if (a.out_step) {
         for (int j = threadIdx.x; j < Q * 3; j += blockDim.x) {
             double s = 0.0;
@@ -1751,7 +1777,7 @@ k_observe(const __grid_constant__ StepArgs<P, Q, R> a)
     for (int64_t base = (int64_t)blockIdx.x * blockDim.x; base < a.N; base += (int64_t)gridDim.x * blockDim.x) {
         if (a.use_win && since_flush + blockDim.x > 65535) {   // 16-bit cells (see phase1_block)
             __syncthreads();
-            flush_window<Q, W>(swin, a.Hnext, ph.Nk, a.win_r0);
+            flush_window<Q, W>(a.Hnext, ph.Nk, a.win_r0, since_flush);
             __syncthreads();
             clear_window<Q, W>(swin);
             __syncthreads();
@@ -1798,7 +1824,7 @@ k_observe(const __grid_constant__ StepArgs<P, Q, R> a)
         }
     }
     __syncthreads();
-    if (a.use_win) flush_window<Q, W>(swin, a.Hnext, ph.Nk, a.win_r0);
+    if (a.use_win) flush_window<Q, W>(a.Hnext, ph.Nk, a.win_r0, since_flush);
     for (int j = threadIdx.x; j < Q * 3; j += blockDim.x) {
         double s = 0.0;
 #pragma unroll
