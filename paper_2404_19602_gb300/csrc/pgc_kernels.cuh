@@ -226,7 +226,8 @@ __device__ __forceinline__ double strided_sum(const double *p, int64_t b0, int64
 
 // The same for 4 values: lane l ends with the sum over the 32 lanes of v[(l >> 3) & 3]; lanes
 // 0, 8, 16, 24 add their sum to the accumulator dst[l >> 3] when that index is below count.
-__device__ __forceinline__ void warp_scatter4_add(const float v[4], float2 *dst, int count, int lane)
+template <typename T>
+__device__ __forceinline__ void warp_scatter4_add(const float v[4], T *dst, int count, int lane)
 {
     float a[2];
 #pragma unroll
@@ -1749,16 +1750,16 @@ k_step(const __grid_constant__ StepArgs<P, Q, R> a1, const __grid_constant__ Ste
 // ------------------------------------------------------------------------------------------
 // Counts go to the block's window as in the streaming kernels (checked cell by cell: an uploaded state
 // may hold anything), FP32 weights come from shared memory, and a node's three sums leave the warp in
-// one reduce-scatter (the same tree as three butterflies).  Counted in the global histogram cell by
-// cell, with indexed parameter-bank weights: 5e5 particles at 36 nodes 235 us; 167 us
-// now.
+// one reduce-scatter (the same tree as three butterflies) and are accumulated in FP64 in both
+// precisions.  Counted in the global histogram cell by cell, with indexed parameter-bank weights: 5e5
+// particles at 36 nodes 235 us; 161 us now.
 template <int P, int Q, typename R>
 __global__ void __launch_bounds__(P1Threads<P, Q, R>::value)
 k_observe(const __grid_constant__ StepArgs<P, Q, R> a)
 {
     constexpr int NW = P1Threads<P, Q, R>::value / 32, W = HistWin<P, Q, R>::W;
     constexpr int row = (P + 1) & ~1;
-    __shared__ typename MomAcc<R>::T smom[NW][Q * 3];
+    __shared__ double smom[NW][Q * 3];
     __shared__ __align__(16) unsigned long long spsi[sizeof(R) == 4 ? Q * row : 2];
     extern __shared__ __align__(16) uint32_t swin[];   // HistWin when a.use_win
     const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;

@@ -36,3 +36,36 @@ def test_sampled_state_and_record_bit_for_bit(row):
     assert hashlib.sha256(np.ascontiguousarray(k).tobytes()).hexdigest() == state
     assert np.concatenate([m["mean"][0], m["var"][0]]).tolist() == values
     assert hashlib.sha256(np.ascontiguousarray(m["nodes"][0]).tobytes()).hexdigest() == nodes
+
+
+def test_fp32_record_is_accumulated_in_fp64():
+    """The warp sums of an FP32 state's record are accumulated in FP64: two energies 2^24 apart, constant over
+    each warp's 32 particles, whose sum of 51 bits comes out exactly (it does not from pairs of FP32
+    numbers)."""
+    from fractions import Fraction
+
+    from paper_2404_19602_gb300 import build, pgc
+
+    if not torch.cuda.is_available():
+        pytest.skip("no CUDA device")
+    build.build()
+    N, big = 1 << 20, 4.0e6   # nm^-1
+    p = W.scaled(W.DET_FP64_1E4, precision="fp32")
+
+    def energy(k):
+        sim = pgc.Simulation(dict(p, N=k.shape[2]), init_khat=k, max_outputs=4)
+        e = sim.moments()["nodes"][0, 0, 2]
+        sim.close()
+        return float(e)
+
+    one = np.zeros((2, 1, 1))
+    ea = energy(one)
+    one[0] = big
+    eb = energy(one)
+    assert np.float32(ea) == ea and np.float32(eb) == eb and 2 ** 21 < eb < 2 ** 22
+    chunks = np.random.default_rng(5).choice(N // 32, 8, replace=False)
+    k = np.zeros((2, 1, N))
+    k[0, 0].reshape(-1, 32)[chunks] = big
+    exact = Fraction(ea) * (N - 8 * 32) + Fraction(eb) * (8 * 32)
+    assert exact == Fraction(float(exact))   # 51 bits: FP64 holds it and every partial sum
+    assert energy(k) == float(exact) / N
