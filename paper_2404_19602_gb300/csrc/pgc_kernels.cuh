@@ -1843,7 +1843,7 @@ k_observe(const __grid_constant__ StepArgs<P, Q, R> a)
 // One band minimum common to several nodes (a random field alone) in FP64: the sampled state does not depend on z,
 // and its higher coefficients and the record's variance over z are the rounding of this kernel and nothing
 // else.  That rounding is part of the output, so it is kept: the energy by the iteration (fd_inverse), projected node
-// by node (FdPerNode; wpsi holds the nodes' own weights).  3e5 particles x 6 nodes: the whole call 12.2 ms with every
+// by node (FdPerNode, k_init_nodes; wpsi holds the nodes' own weights).  3e5 particles x 6 nodes: the whole call 12.2 ms with every
 // node inverted, 2.3 ms with one inversion per particle (0.6 ms from the table, with another rounding).
 template <int Q, typename R> struct FdPerNode {
     static constexpr bool possible = Q > 1 && sizeof(R) == 8;
@@ -1852,7 +1852,6 @@ template <int Q, typename R> struct FdPerNode {
 template <int P, int Q>
 struct InitArgs {
     int32_t ng;        // distinct band minima
-    int32_t per_node;  // FdPerNode
     double wpsi[Q * P];
     double eps0[Q];
     double ratio[Q], y0[Q];   // G(w0_q) / Gmax and (eps0_q / kT)^2 (the table of pgc_fd.cuh)
@@ -1877,30 +1876,6 @@ k_init(const __grid_constant__ InitArgs<P, Q> ia, R *khat)
         const double ue = u01<double>(r.x), uth = u01<double>(r.y);
         double s, c;
         sincos(2.0 * kPi * uth, &s, &c);
-        if constexpr (FdPerNode<Q, R>::possible) {
-            if (ia.per_node) {
-                const double e0 = ia.eps0[0], eps = fd_inverse(e0, ia.mu, ia.kT, ue), rr = eps * eps - e0 * e0;
-                const double km = (rr > 0.0) ? sqrt(rr) / ia.hvF : 0.0;
-                const double kx = km * c, ky = km * s;
-                double hx[P], hy[P];
-#pragma unroll
-                for (int h = 0; h < P; ++h) { hx[h] = 0.0; hy[h] = 0.0; }
-#pragma unroll 1
-                for (int q = 0; q < Q; ++q) {
-#pragma unroll
-                    for (int h = 0; h < P; ++h) {
-                        hx[h] += ia.wpsi[q * P + h] * kx;
-                        hy[h] += ia.wpsi[q * P + h] * ky;
-                    }
-                }
-#pragma unroll
-                for (int h = 0; h < P; ++h) {
-                    khat[(int64_t)h * ia.ld + i] = (R)(ia.strang ? hx[h] + ia.dhalf[h] : hx[h]);
-                    khat[(int64_t)(P + h) * ia.ld + i] = (R)hy[h];
-                }
-                continue;
-            }
-        }
         double hk[P];
 #pragma unroll
         for (int h = 0; h < P; ++h) hk[h] = 0.0;
@@ -1924,6 +1899,38 @@ k_init(const __grid_constant__ InitArgs<P, Q> ia, R *khat)
             const double hx = hk[h] * c, hy = hk[h] * s;
             khat[(int64_t)h * ia.ld + i] = (R)(ia.strang ? hx + ia.dhalf[h] : hx);
             khat[(int64_t)(P + h) * ia.ld + i] = (R)hy;
+        }
+    }
+}
+
+// The sampler of an FdPerNode ensemble (a kernel of its own: k_init has no registers for it).
+template <int P, int Q, typename R>
+__global__ void __launch_bounds__(128)
+k_init_nodes(const __grid_constant__ InitArgs<P, Q> ia, R *khat)
+{
+    for (int64_t i = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; i < ia.N; i += (int64_t)gridDim.x * blockDim.x) {
+        const U4 r = philox4x32_10((uint32_t)i, ia.stream_id, 0u, 0x10000u, ia.key0, ia.key1);
+        const double ue = u01<double>(r.x), uth = u01<double>(r.y);
+        double s, c;
+        sincos(2.0 * kPi * uth, &s, &c);
+        const double e0 = ia.eps0[0], eps = fd_inverse(e0, ia.mu, ia.kT, ue), rr = eps * eps - e0 * e0;
+        const double km = (rr > 0.0) ? sqrt(rr) / ia.hvF : 0.0;
+        const double kx = km * c, ky = km * s;
+        double hx[P], hy[P];
+#pragma unroll
+        for (int h = 0; h < P; ++h) { hx[h] = 0.0; hy[h] = 0.0; }
+#pragma unroll 1
+        for (int q = 0; q < Q; ++q) {
+#pragma unroll
+            for (int h = 0; h < P; ++h) {
+                hx[h] += ia.wpsi[q * P + h] * kx;
+                hy[h] += ia.wpsi[q * P + h] * ky;
+            }
+        }
+#pragma unroll
+        for (int h = 0; h < P; ++h) {
+            khat[(int64_t)h * ia.ld + i] = (R)(ia.strang ? hx[h] + ia.dhalf[h] : hx[h]);
+            khat[(int64_t)(P + h) * ia.ld + i] = (R)hy[h];
         }
     }
 }

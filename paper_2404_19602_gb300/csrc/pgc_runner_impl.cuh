@@ -88,8 +88,7 @@ public:
         args_.stream_id = b.stream_id;
         int of[Q];
         init_.ng = fd_groups(t.eps0.data(), Q, t.wpsi.data(), P, init_.eps0, init_.wpsi, of);
-        init_.per_node = FdPerNode<Q, R>::value(init_.ng) ? 1 : 0;
-        if (init_.per_node) std::copy(t.wpsi.begin(), t.wpsi.begin() + Q * P, init_.wpsi);
+        if (FdPerNode<Q, R>::value(init_.ng)) std::copy(t.wpsi.begin(), t.wpsi.begin() + Q * P, init_.wpsi);
         init_.mu = t.mu;
         init_.kT = t.kT;
         init_.hvF = t.hvF;
@@ -143,7 +142,14 @@ public:
 
     cudaError_t init_sample(cudaStream_t s) override
     {
-        if (b_.fdtab && !init_.per_node) {
+        const int blocks = (int)std::min<int64_t>((b_.N + 127) / 128, 8192);
+        if constexpr (FdPerNode<Q, R>::possible)
+            if (FdPerNode<Q, R>::value(init_.ng)) {
+                k_init_nodes<P, Q, R><<<blocks, 128, 0, s>>>(init_, args_.khat);
+                count_launch();
+                return cudaGetLastError();
+            }
+        if (b_.fdtab) {
             init_.fd = fd_plan(init_.eps0, init_.ng, init_.mu, init_.kT, init_.ratio);
             for (int q = 0; q < init_.ng; ++q) { const double w0 = init_.eps0[q] / init_.kT; init_.y0[q] = w0 * w0; }
             if (init_.fd.n > 0) {
@@ -152,7 +158,6 @@ public:
                 init_.fd.tab = b_.fdtab;
             }
         }
-        int blocks = (int)std::min<int64_t>((b_.N + 127) / 128, 8192);
         k_init<P, Q, R><<<blocks, 128, 0, s>>>(init_, args_.khat);
         count_launch();
         return cudaGetLastError();
