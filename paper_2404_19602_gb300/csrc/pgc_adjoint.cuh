@@ -359,7 +359,7 @@ __device__ __forceinline__ void replay_events(const Phys<R> &ph, const Nodes<P, 
                 l_out[s] = 6;
                 if (q >= Q) continue;
                 R g[6];
-                rates6(ph, kx[s], ky[s], nd.eps0[q], g);
+                rates6<false>(ph, kx[s], ky[s], nd.eps0[q], g);
                 int l = 6;
                 R cum = (R)0;
 #pragma unroll
@@ -389,7 +389,9 @@ __device__ __forceinline__ void replay_events(const Phys<R> &ph, const Nodes<P, 
             const int q = r + s * G;
             if (q >= Q) continue;
             R g[6];
-            rates6(ph, kx[s], ky[s], nd.eps0[q], g);
+            // (rounded as this replay's selection always was: a mechanism boundary hit to the last bit goes
+            // one way in ~1e-8 of the events, and one event moves a gradient of 5e5 particles by 1e-6)
+            rates6<false>(ph, kx[s], ky[s], nd.eps0[q], g);
             int l = 6;
             R cum = (R)0;
 #pragma unroll

@@ -232,13 +232,12 @@ __device__ __forceinline__ R edge_T(const Phys<R> &ph, R beta, R c)
 }
 
 // Rates of the six mechanisms of Eq. (20) at one state (Appendix A closed forms).  Returns the sum.
-// (In eps^2 = eps0^2 + (hvF |k|)^2 the first product is fused: written out, so that the adjoint's replay selects
-// the mechanisms that the forward run selected.)
-template <typename R>
+// E0FUSED: which product of eps^2 = eps0^2 + (hvF |k|)^2 is fused.
+template <bool E0FUSED = true, typename R = float>
 __device__ __forceinline__ R rates6(const Phys<R> &ph, R kx, R ky, R eps0, R g[6])
 {
     const R kk = sum2(kx, kx, ky, ky);
-    const R eps = rsqrt_<R>(sum2(eps0, eps0, ph.hvF2, kk));
+    const R eps = rsqrt_<R>(E0FUSED ? sum2(eps0, eps0, ph.hvF2, kk) : sum2(ph.hvF2, kk, eps0, eps0));
     const uint32_t m = ph.mech;
     g[0] = (m & 1u) ? ph.Cac * eps : (R)0;
     g[1] = ((m & 2u) && (eps - ph.hwO - eps0 > (R)0)) ? ph.COm * (eps - ph.hwO) : (R)0;
