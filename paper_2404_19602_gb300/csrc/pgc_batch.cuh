@@ -146,7 +146,7 @@ k_phase1_batch(const __grid_constant__ BatchArgs<P, Q, R> a)
             n_aside = 0;
         }
         __syncthreads();
-        if (a.use_win) flush_window<Q, HistWin<P, Q, R>::batchW>(t.Hnext, a.ph.Nk, a.win_r0, p1 - p0);
+        if (a.use_win) flush_quads<Q, HistWin<P, Q, R>::batchW>(swin, t.Hnext, a.ph.Nk, a.win_r0);
         if (out)
             for (int j = threadIdx.x; j < Q * 3; j += blockDim.x) {
                 double s = 0.0;

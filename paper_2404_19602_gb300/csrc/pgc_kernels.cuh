@@ -357,10 +357,9 @@ __device__ __forceinline__ F2 f2_add_rd(F2 a, F2 b)
 // row - r0 and 4 (column - r0) + fraction.  Three packed operations and a multiply-add where two
 // additions, two multiplications, two conversions, the bounds checks and the word and shift
 // arithmetic were ~20.  A particle whose |k| stays inside the window's circle at every node (kk_in, from
-// the majorant's kkmax that the screen needs anyway) takes no per-node check at all.  Measured: the
-// streaming kernel at 4e6 particles x 36 nodes 465 -> 237 us in the first 50 steps, 487 -> 260 us after
-// 3000 (one step in ten with moments); the batched kernel at 32 cases, 1.3e7 particles x 6 nodes
-// 355 -> 246 and 388 -> 269 us; instructions issued bound both.
+// the majorant's kkmax that the screen needs anyway) takes no per-node check at all.  Instructions
+// issued bound the streaming kernel: at 4e6 particles x 36 nodes 468 us a launch with the checks, 250 without (481
+// and 256 after 2000 steps; one step in ten with moments).
 template <int W>
 __device__ __forceinline__ uint32_t window_code(float kx, float ky, unsigned long long lk2, F2 inv2, F2 magic2)
 {
@@ -1049,48 +1048,53 @@ __device__ __forceinline__ void clear_window(uint32_t *swin)
         reinterpret_cast<uint4 *>(swin)[j] = make_uint4(0u, 0u, 0u, 0u);
 }
 
-// Add it to the global histogram, one add per non-empty cell and node.  A lane takes one word, so that a warp's adds
-// fall on 32 cells side by side, four sectors of L2: with four cells a lane they fell on sixteen, and the
-// fuller the window the more the flush was the step (1e6 particles x 6 nodes, us a step: 240 cells 33.6 -> 32.2, after
-// 3000 steps 38.5 -> 35.9; 480 cells 48.2 -> 36.4; 600 cells 57 -> 41).  A sparse window at 36 nodes (the
-// block has counted fewer than kSparseWindow particles) is looked at four words a load all the same, since there the
-// words looked at are the cost (2e5 particles, 1300 a block: 27.5 us a launch, 29.0 word by word; at 4e6 the
-// two are equal).  Not inlined: the streaming loop has no register to spare for it.
-constexpr int kSparseWindow = 2000;
+// Add it to the global histogram, one add per non-empty cell and node; flush_quads with four cells a lane, which
+// passes over empty words fastest, flush_window word by word, so that a warp's adds fall on 32 cells side
+// by side, four sectors of L2 instead of sixteen.  The fuller the window the more the adds are the step (1e6 particles
+// x 6 nodes, us a step, quads / words: 240 cells 33.5 / 32.4, after 3000 steps 38.4 / 36.0; 480 cells 48.2 /
+// 36.4; 600 cells 57 / 41); a window that has counted fewer than kSparseWindow particles on a grid of fewer than
+// kFineGrid cells is mostly empty (36 nodes, 2e5 particles, 1300 a block, us a launch: 240 cells 27.5 / 29.0;
+// 6 nodes, 3e5 particles, 1024 a block, us a step: 480 cells 25.1 / 22.6), as are those of the batch's tiles.
+// Not inlined: the streaming loop has no register to spare for it.
+constexpr int kSparseWindow = 2000, kFineGrid = 400;
+template <int Q, int W>
+__device__ __forceinline__ void flush_quads(const uint32_t *swin, uint32_t *Hnext, int Nk, int win_r0)
+{
+    const int64_t NN = (int64_t)Nk * Nk;
+    for (int j = threadIdx.x; j < (Q + 1) / 2 * (W * W / 4); j += blockDim.x) {
+        const uint4 v4 = reinterpret_cast<const uint4 *>(swin)[j];
+        if (!(v4.x | v4.y | v4.z | v4.w)) continue;
+        const int p = j / (W * W / 4), w = j % (W * W / 4);
+        uint32_t *base = Hnext + (int64_t)(2 * p) * NN + (int64_t)(w / (W / 4) + win_r0) * Nk + 4 * (w % (W / 4)) + win_r0;
+        const uint32_t v[4] = {v4.x, v4.y, v4.z, v4.w};
+#pragma unroll
+        for (int c = 0; c < 4; ++c) {
+            if (v[c] & 0xffffu) atomicAdd(base + c, v[c] & 0xffffu);
+            if (v[c] >> 16) atomicAdd(base + NN + c, v[c] >> 16);
+        }
+    }
+}
+
 template <int Q, int W>
 __device__ __noinline__ void flush_window(uint32_t *Hnext, int Nk, int win_r0, int64_t counted)
 {
     extern __shared__ __align__(16) uint32_t swin[];
+    if (counted < kSparseWindow && Nk < kFineGrid) return flush_quads<Q, W>(swin, Hnext, Nk, win_r0);
     constexpr uint32_t n = (Q + 1) / 2 * W * W, U = Q > 6 ? 8 : 4;
     const uint32_t NN = (uint32_t)Nk * Nk, pair = 2 * NN - W * (uint32_t)Nk;   // (a histogram of all nodes has < 2^32 cells)
     uint32_t *base = Hnext + win_r0 * (Nk + 1);
-    auto cell = [&](uint32_t j) {
-        const uint32_t r = j / W, p = r / W;   // row of all pairs' windows, node pair
-        return base + (size_t)(p * pair + r * (uint32_t)Nk + (j - r * W));
-    };
-    auto add = [&](uint32_t *h, uint32_t v) {
-        if (v & 0xffffu) atomicAdd(h, v & 0xffffu);
-        if (v >> 16) atomicAdd(h + NN, v >> 16);
-    };
-    if (Q == 36 && counted < kSparseWindow) {
-        for (uint32_t j = threadIdx.x; j < n / 4; j += blockDim.x) {
-            const uint4 v = reinterpret_cast<const uint4 *>(swin)[j];
-            if (!(v.x | v.y | v.z | v.w)) continue;
-            uint32_t *h = cell(4 * j);
-            add(h, v.x);
-            add(h + 1, v.y);
-            add(h + 2, v.z);
-            add(h + 3, v.w);
-        }
-        return;
-    }
     for (uint32_t j0 = threadIdx.x; j0 < n; j0 += U * blockDim.x) {
         uint32_t v[U];
 #pragma unroll
         for (uint32_t u = 0; u < U; ++u) v[u] = j0 + u * blockDim.x < n ? swin[j0 + u * blockDim.x] : 0u;
 #pragma unroll
-        for (uint32_t u = 0; u < U; ++u)
-            if (v[u]) add(cell(j0 + u * blockDim.x), v[u]);
+        for (uint32_t u = 0; u < U; ++u) {
+            if (!v[u]) continue;
+            const uint32_t j = j0 + u * blockDim.x, r = j / W, p = r / W;   // row of all pairs' windows, node pair
+            uint32_t *h = base + (size_t)(p * pair + r * (uint32_t)Nk + (j - r * W));
+            if (v[u] & 0xffffu) atomicAdd(h, v[u] & 0xffffu);
+            if (v[u] >> 16) atomicAdd(h + NN, v[u] >> 16);
+        }
     }
 }
 
