@@ -198,7 +198,7 @@ pgc_status pgc_step(pgc_ctx *ctx, int64_t n_steps, int32_t moments_every);
  * and precision except P = 21, Q = 36 in FP64 (PGC_EUNSUPPORTED: the fused kernel's two argument
  * blocks exceed the kernel-parameter space).  On by default when P * Q <= 64; until the first call
  * of this function, FP32 contexts of the larger one-dimensional shapes with at most 2e5 particles
- * also take it in pgc_step calls without moment records. */
+ * and 3e6 node values (particles times nodes) also take it in pgc_step calls without moment records. */
 pgc_status pgc_set_pipeline(pgc_ctx *ctx, int32_t on);
 
 /* Copy the recorded time series to the host (synchronizes).  Any pointer may be NULL.

@@ -791,11 +791,13 @@ pgc_status pgc_init(const pgc_config *cfg, void *d_state, void *d_hist, void *d_
     // most resident blocks for the whole launch: measured slower, so off by default there
     ctx->pipeline = (ctx->run->fused() && L.P * L.Q <= 64) ? 1 : 0;
     // The larger one-dimensional shapes: two launches of one latency chain each at the sizes of the error
-    // study, so fused is faster up to 2e5 particles (us a step, two launches / fused: 21 nodes 32.3 /
-    // 26.2 at 1e4, 69.5 / 64.5 at 2e5, 227 / 236 at 1e6; 9 nodes 23.6 / 17.6, 41.1 / 34.3, 108 / 113).  Only
-    // for calls without moment records: the states are the same bit for bit, the records' FP32 warp
+    // study, so fused is faster while the particles are few (us a step, two launches / fused: 21 nodes 31.0 /
+    // 25.1 at 1e4, 46.0 / 45.9 at 1e5, 65.3 / 69.7 at 2e5; 13 nodes 37.0 / 29.7 at 1e5, 50.3 / 44.6 at 2e5, 71.2 / 71.2
+    // at 4e5; 9 nodes 24.0 / 18.2 at 1e4, 44.2 / 37.5 at 2e5, 59.5 / 59.5 at 4e5): up to 2e5 particles and 3e6 node values.
+    // Only for calls without moment records: the states are the same bit for bit, the records' FP32 warp
     // sums are grouped differently.
-    ctx->pipeline_auto = (!ctx->pipeline && ctx->run->fused() && L.d == 1 && cfg->precision == PGC_FP32 && cfg->n_particles <= 200000) ? 1 : 0;
+    ctx->pipeline_auto = (!ctx->pipeline && ctx->run->fused() && L.d == 1 && cfg->precision == PGC_FP32 && cfg->n_particles <= 200000 &&
+                          cfg->n_particles * L.Q <= 3000000) ? 1 : 0;
     if (cfg->tc_proj != PGC_TC_OFF) {
         if ((e = ctx->run->set_tc(cfg->tc_proj)) != cudaSuccess) {
             delete ctx->run; delete ctx;
