@@ -12,7 +12,7 @@
 //                 drift term -d(dhat)/d(theta).lambda.  Without a moment term it reads the bitmap and
 //                 the planes of lambda that the drift term needs, nothing else;
 //   k_adj_collide (queued, lanes <-> nodes as in the forward collider kernel): replays the event
-//                 chain of step n bit for bit, then applies the transposed Jacobians of the
+//                 chain of step n (FP32: but for one event in ~3e6, see replay_events), then applies the transposed Jacobians of the
 //                 projection, the final-state maps h^l and the reconstruction, event by event from
 //                 the last (each event's input state is recomputed by replaying from the start),
 //                 and adds the drift term.
@@ -302,9 +302,14 @@ __device__ void fs_jacobian(const Phys<R> &ph, int l, R kx, R ky, EventAngles<R>
     J[2] = st * M0 + ct * M2; J[3] = st * M1 + ct * M3;
 }
 
-// Replays the collision loop of collide_particle for particle i (same operations, same group
-// layout; an event that changes no node leaves the coefficients, rates and majorant untouched)
-// for at most `stop` events; on return cx/cy/kx/ky hold the state before event `stop` (or the
+// Replays the collision loop of collide_particle for particle i (same group layout, same operations but for
+// one rounding: eps^2 of the rates that the mechanism is selected by has its other product fused,
+// rates6<false>).  In FP32 a target within the last bit of a mechanism's boundary then selects the neighbour of the
+// forward run's choice: 3 of 9.4 million events at 6 nodes (FP64: none).  Such a chain moves a gradient by 1e-9
+// to 1.5e-6 of its size, far below the ensemble's sampling noise.  Selecting by rates6<true> moves the gradients of
+// the runs that hold one by as much (3 of 44): beyond the 1e-9 to which the adjoint's results are held from
+// one build to the next, so the rounding stays.  (An event that changes no node leaves the
+// coefficients, rates and majorant untouched.)  Replays at most `stop` events; on return cx/cy/kx/ky hold the state before event `stop` (or the
 // final state), and *nev the number of events the loop would run.  The mechanism of every node
 // at event `stop` is returned in l_out[] (6 = unchanged).  rec(e, s, kx, ky, l, r) is called for every
 // event e applied and node slot s with the node value before it and its mechanism (6 = unchanged).
@@ -389,8 +394,7 @@ __device__ __forceinline__ void replay_events(const Phys<R> &ph, const Nodes<P, 
             const int q = r + s * G;
             if (q >= Q) continue;
             R g[6];
-            // (rounded as this replay's selection always was: a mechanism boundary hit to the last bit goes
-            // one way in ~1e-8 of the events, and one event moves a gradient of 5e5 particles by 1e-6)
+            // (the rounding of the selection: see above)
             rates6<false>(ph, kx[s], ky[s], nd.eps0[q], g);
             int l = 6;
             R cum = (R)0;
