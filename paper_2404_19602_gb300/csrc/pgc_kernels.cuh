@@ -588,10 +588,16 @@ __device__ __forceinline__ void recon_stored(const Nodes<P, Q, R> &nd, int q, co
 
 // group velocity (units of vF) and energy at one node (Sec. 2).  The warp partial sums are
 // taken in R (FP32 in the production mode, FP64 in the FP64 mode) and accumulated in FP64.
-template <typename R>
+// In FP32 the contraction is written out (which products are rounded: left to the compiler it follows the
+// surrounding code, and a record of a thousand particles moves by 1e-8); the one-node shape keeps the
+// compiler's, which is another there.
+template <int Q, typename R>
 __device__ __forceinline__ void observe(const Phys<R> &ph, R kx, R ky, R eps0, R &vx, R &vy, R &e)
 {
-    const R eps = rsqrt_<R>(ph.hvF2 * (kx * kx + ky * ky) + eps0 * eps0);
+    R s2;
+    if constexpr (sizeof(R) == 4 && Q > 1) s2 = fma_rn(eps0, eps0, mul_rn(ph.hvF2, fma_rn(ky, ky, mul_rn(kx, kx))));
+    else s2 = ph.hvF2 * (kx * kx + ky * ky) + eps0 * eps0;
+    const R eps = rsqrt_<R>(s2);
     vx = ph.hvF * kx / eps;
     vy = ph.hvF * ky / eps;
     e = eps;
@@ -977,7 +983,7 @@ __device__ __forceinline__ void phase1_pass(const Phys<R> &ph, const Nodes<P, Q,
                     if (finished[e]) {
                         float kx, ky, a1, a2, a3;
                         recon_node(ndb, q, cx[e], cy[e], kx, ky);
-                        observe(ph, kx - nd.xs[q], ky, nd.eps0[q], a1, a2, a3);
+                        observe<Q>(ph, kx - nd.xs[q], ky, nd.eps0[q], a1, a2, a3);
                         s[0] += a1; s[1] += a2; s[2] += a3;
                     }
                 warp_scatter4_add(s, smom_warp + q * 3, 3, lane);
@@ -991,7 +997,7 @@ __device__ __forceinline__ void phase1_pass(const Phys<R> &ph, const Nodes<P, Q,
                     if (finished[e]) {
                         R kx, ky, a1, a2, a3;
                         recon_node(ndb, q, cx[e], cy[e], kx, ky);
-                        observe(ph, kx - nd.xs[q], ky, nd.eps0[q], a1, a2, a3);
+                        observe<Q>(ph, kx - nd.xs[q], ky, nd.eps0[q], a1, a2, a3);
                         vx += a1; vy += a2; en += a3;
                     }
                 vx = warp_sum(vx);
@@ -1561,7 +1567,7 @@ __device__ __forceinline__ void collide_particle(const Phys<R> &ph, const Nodes<
         else ++cnt.oog;
         if (t.out_step) {
             R vx, vy, e;
-            observe(ph, x - nd.xs[q], y, nd.eps0[q], vx, vy, e);
+            observe<Q>(ph, x - nd.xs[q], y, nd.eps0[q], vx, vy, e);
             atomicAdd(&t.mom[q * 3 + 0], (double)vx);
             atomicAdd(&t.mom[q * 3 + 1], (double)vy);
             atomicAdd(&t.mom[q * 3 + 2], (double)e);
@@ -1608,7 +1614,7 @@ __device__ __forceinline__ void collide_particle(const Phys<R> &ph, const Nodes<
                 if (t.out_next) {
                     R x, y, vx, vy, e;
                     recon_node(nd, q, cx, cy, x, y);
-                    observe(ph, x - nd.xs[q], y, nd.eps0[q], vx, vy, e);
+                    observe<Q>(ph, x - nd.xs[q], y, nd.eps0[q], vx, vy, e);
                     atomicAdd(&t.momN[q * 3 + 0], (double)vx);
                     atomicAdd(&t.momN[q * 3 + 1], (double)vy);
                     atomicAdd(&t.momN[q * 3 + 2], (double)e);
@@ -1815,7 +1821,7 @@ k_observe(const __grid_constant__ StepArgs<P, Q, R> a)
                     else
                         atomicAdd(&a.Hnext[(int64_t)q * NN + r * ph.Nk + l], 1u);
                 }
-                observe(ph, kx - nd.xs[q], ky, nd.eps0[q], o[0], o[1], o[2]);
+                observe<Q>(ph, kx - nd.xs[q], ky, nd.eps0[q], o[0], o[1], o[2]);
             }
             if constexpr (sizeof(R) == 4) {
                 warp_scatter4_add(o, smom[warp] + q * 3, 3, lane);
